@@ -104,64 +104,72 @@ __device__ __forceinline__ void collide27(R g[Q27], const Relax27<R> &p)
     R drho = g[0];
 #pragma unroll
     for (int k = 0; k < 13; ++k) drho += s[k];
-    R j[3] = {R(0), R(0), R(0)};
-#pragma unroll
-    for (int k = 0; k < 13; ++k) {
-        const int q = 2 * k + 1;
-        if (CX(q)) j[0] += R(CX(q)) * d[k];
-        if (CY(q)) j[1] += R(CY(q)) * d[k];
-        if (CZ(q)) j[2] += R(CZ(q)) * d[k];
-    }
     R P = R(1), u[3], du[3] = {R(0), R(0), R(0)};
     constexpr bool COMP = compensated_v<R, ONE_ROUNDING> && !RHO0;
-    if (RHO0) {
-        P = R(1) + drho;
-        const R inv = R(1) / P;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) u[i] = (j[i] + p.half_a[i]) * inv;
-    } else if (COMP) {
+    // momentum; pair k < 3 is the face pair of axis k (c = +e_k) and starts the sum
+    R j[3] = {d[0], d[1], d[2]};
+    if (COMP) {
         // compensated momentum, as CellEq does for D3Q19 (FP32 storage): u is
         // rounded, du = (j + a/2) - u exactly, and the face pair of each axis
-        // (k = 0, 1, 2: c = +e_x, +e_y, +e_z) takes du out of its
-        // antisymmetric non-equilibrium, so the momentum balance stays exact
-        R hi[3] = {d[0], d[1], d[2]}, lo[3] = {R(0), R(0), R(0)};
+        // takes du out of its antisymmetric non-equilibrium, so the momentum
+        // balance stays exact
+        R lo[3] = {R(0), R(0), R(0)};
 #pragma unroll
         for (int k = 3; k < 13; ++k) {
             const int q = 2 * k + 1;
-            if (CX(q) != 0) two_sum_acc(hi[0], lo[0], CX(q) > 0 ? d[k] : -d[k]);
-            if (CY(q) != 0) two_sum_acc(hi[1], lo[1], CY(q) > 0 ? d[k] : -d[k]);
-            if (CZ(q) != 0) two_sum_acc(hi[2], lo[2], CZ(q) > 0 ? d[k] : -d[k]);
+            if (CX(q) != 0) two_sum_acc(j[0], lo[0], CX(q) > 0 ? d[k] : -d[k]);
+            if (CY(q) != 0) two_sum_acc(j[1], lo[1], CY(q) > 0 ? d[k] : -d[k]);
+            if (CZ(q) != 0) two_sum_acc(j[2], lo[2], CZ(q) > 0 ? d[k] : -d[k]);
         }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            u[i] = hi[i];
+            u[i] = j[i];
             two_sum_acc(u[i], lo[i], p.half_a[i]);
             du[i] = lo[i];
         }
     } else {
 #pragma unroll
+        for (int k = 3; k < 13; ++k) {
+            const int q = 2 * k + 1;
+            if (CX(q)) j[0] = CX(q) > 0 ? j[0] + d[k] : j[0] - d[k];
+            if (CY(q)) j[1] = CY(q) > 0 ? j[1] + d[k] : j[1] - d[k];
+            if (CZ(q)) j[2] = CZ(q) > 0 ? j[2] + d[k] : j[2] - d[k];
+        }
+#pragma unroll
         for (int i = 0; i < 3; ++i) u[i] = j[i] + p.half_a[i];
+        if (RHO0) {
+            P = R(1) + drho;
+            const R inv = R(1) / P;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) u[i] = mul(u[i], inv);
+        }
     }
-    const R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const R base = drho - R(1.5) * P * uu;
-    g[0] = fma(-p.wp, g[0] - p.w[0] * base, g[0]);
+    const R uu = mad(u[2], u[2], mad(u[1], u[1], mul(u[0], u[0])));
+    const R base = mad(RHO0 ? mul(R(-1.5f), P) : R(-1.5f), uu, drho);
+    g[0] = mad(-p.wp, mad(-p.w[0], base, g[0]), g[0]);
+    R K[4], A[4], wb[4];
+#pragma unroll
+    for (int c = 1; c < 4; ++c) {
+        K[c] = RHO0 ? mul(P, p.K[c]) : p.K[c];
+        A[c] = RHO0 ? mul(P, p.A[c]) : p.A[c];
+        wb[c] = mul(p.w[c], base);
+    }
 #pragma unroll
     for (int k = 0; k < 13; ++k) {
         const int q = 2 * k + 1;
         const int cls = NORM2(q);
-        const R cu = R(CX(q)) * u[0] + R(CY(q)) * u[1] + R(CZ(q)) * u[2];
-        const R sym = p.w[cls] * base + (P * p.K[cls]) * (cu * cu);
-        const R nsym = fma(R(-2), sym, s[k]);
-        R nasym = fma(-(P * p.A[cls]), cu, d[k]);
+        const R cu = along(CX(q), CY(q), CZ(q), u);
+        const R sym = mad(K[cls], mul(cu, cu), wb[cls]);
+        const R nsym = mad(R(-2), sym, s[k]);
+        R nasym = mad(-A[cls], cu, d[k]);
         if (COMP && k < 3) nasym -= du[k];
-        const R b = fma(p.hm, nasym, -p.force[k]);
+        const R b = mad(p.hm, nasym, -p.force[k]);
         if (ONE_ROUNDING) {
-            g[q] = g[q] - fma(p.hp, nsym, b);
-            g[q + 1] = g[q + 1] - fma(p.hp, nsym, -b);
+            g[q] = g[q] - mad(p.hp, nsym, b);
+            g[q + 1] = g[q + 1] - mad(p.hp, nsym, -b);
         } else {
-            const R a1 = p.hp * nsym;
-            g[q] = (g[q] - a1) - b;
-            g[q + 1] = (g[q + 1] - a1) + b;
+            g[q] = mad(-p.hp, nsym, g[q]) - b;
+            g[q + 1] = mad(-p.hp, nsym, g[q + 1]) + b;
         }
     }
 }

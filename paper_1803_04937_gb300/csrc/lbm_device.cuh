@@ -345,6 +345,17 @@ __device__ __forceinline__ void collide(R g[Q], const Coll<R> &p)
 
 // ---------------------------------------------------------------- lean collision (step kernels)
 
+// Products and fused multiply-adds of the collision, written out (plain
+// products are never left to be contracted), so that every kernel rounds a
+// cell's update alike.
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+
+template <typename R> __device__ __forceinline__ R third() { return R(1.0f / 3.0f); }
+template <> __device__ __forceinline__ double third<double>() { return 1.0 / 3.0; }
+
 // Per-launch constants of the collision, folded so that a cell update needs
 // few instructions.  With P = rho0 (1, or rho when rho0 = rho) and base =
 // drho - 3/2 P u^2, the symmetric (even) equilibrium part of a pair is
@@ -408,8 +419,20 @@ __device__ __forceinline__ void two_sum_acc(R &hi, R &lo, R v)
     hi = s;
 }
 
+// c_q . u of a lattice direction (c: its components, -1, 0 or 1) without the
+// products by 0 and +-1, which the compiler may not drop by itself.
+template <typename R>
+__device__ __forceinline__ R along(int cx, int cy, int cz, const R u[3])
+{
+    R r = cx ? (cx > 0 ? u[0] : -u[0]) : (cy ? (cy > 0 ? u[1] : -u[1]) : (cz > 0 ? u[2] : -u[2]));
+    if (cx && cy) r = cy > 0 ? r + u[1] : r - u[1];
+    if ((cx || cy) && cz) r = cz > 0 ? r + u[2] : r - u[2];
+    return r;
+}
+
 // Moments and symmetric-equilibrium bases of one cell, shared by the step and
-// the adjoint.  s[k], d[k]: sum and difference of pair k (q = 2k+1, q + 1).
+// the adjoint.  s[k], d[k]: sum and difference of pair
+// k (q = 2k+1, q + 1).
 //
 // COMP (rho0 = 1 only): the momentum is summed with TwoSum, and du = (j +
 // a/2) - u, the part of the exact velocity that rounding u drops, is kept.
@@ -437,36 +460,34 @@ struct CellEq {
             d[k] = g[2 * k + 1] - g[2 * k + 2];
         }
         const R drho = g[0] + (((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7])) + s[8]);
-        R j[3] = {R(0), R(0), R(0)};
+        // momentum: pair k < 3 is the face pair of axis k (c = +e_k) and starts the sum
+        R j[3] = {d[0], d[1], d[2]};
+        if (RHO0_IS_RHO || !COMP) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int q = 2 * k + 1;
-            if (CX(q) > 0) j[0] += d[k];
-            if (CX(q) < 0) j[0] -= d[k];
-            if (CY(q) > 0) j[1] += d[k];
-            if (CY(q) < 0) j[1] -= d[k];
-            if (CZ(q) > 0) j[2] += d[k];
-            if (CZ(q) < 0) j[2] -= d[k];
+            for (int k = 3; k < 9; ++k) {
+                const int q = 2 * k + 1;
+                if (CX(q) != 0) j[0] = CX(q) > 0 ? j[0] + d[k] : j[0] - d[k];
+                if (CY(q) != 0) j[1] = CY(q) > 0 ? j[1] + d[k] : j[1] - d[k];
+                if (CZ(q) != 0) j[2] = CZ(q) > 0 ? j[2] + d[k] : j[2] - d[k];
+            }
         }
-        P = R(1);
         if (RHO0_IS_RHO) {
             P = R(1) + drho;
             const R inv = R(1) / P;
 #pragma unroll
-            for (int i = 0; i < 3; ++i) u[i] = (j[i] + p.half_a[i]) * inv;
+            for (int i = 0; i < 3; ++i) u[i] = mul(j[i] + p.half_a[i], inv);
         } else if (COMP) {
-            // pair k < 3 is the face pair of axis k (c = +e_k): it starts the sum
-            R hi[3] = {d[0], d[1], d[2]}, lo[3] = {R(0), R(0), R(0)};
+            R lo[3] = {R(0), R(0), R(0)};
 #pragma unroll
             for (int k = 3; k < 9; ++k) {
                 const int q = 2 * k + 1;
-                if (CX(q) != 0) two_sum_acc(hi[0], lo[0], CX(q) > 0 ? d[k] : -d[k]);
-                if (CY(q) != 0) two_sum_acc(hi[1], lo[1], CY(q) > 0 ? d[k] : -d[k]);
-                if (CZ(q) != 0) two_sum_acc(hi[2], lo[2], CZ(q) > 0 ? d[k] : -d[k]);
+                if (CX(q) != 0) two_sum_acc(j[0], lo[0], CX(q) > 0 ? d[k] : -d[k]);
+                if (CY(q) != 0) two_sum_acc(j[1], lo[1], CY(q) > 0 ? d[k] : -d[k]);
+                if (CZ(q) != 0) two_sum_acc(j[2], lo[2], CZ(q) > 0 ? d[k] : -d[k]);
             }
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                u[i] = hi[i];
+                u[i] = j[i];
                 two_sum_acc(u[i], lo[i], p.half_a[i]);
                 du[i] = lo[i];
             }
@@ -475,21 +496,24 @@ struct CellEq {
             for (int i = 0; i < 3; ++i) u[i] = j[i] + p.half_a[i];
         }
 #pragma unroll
-        for (int i = 0; i < 3; ++i) u2[i] = u[i] * u[i];
-        uu = u2[0] + u2[1] + u2[2];
+        for (int i = 0; i < 3; ++i) u2[i] = mul(u[i], u[i]);
+        uu = (u2[0] + u2[1]) + u2[2];
         R k0 = p.k0, kf = p.kf, ke = p.ke;
         Kf = p.Kf;
         Ke = p.Ke;
         Af = p.Af;
         Ae = p.Ae;
+        R h = R(-1.5);  // -3/2 P
         if (RHO0_IS_RHO) {
-            k0 *= P; kf *= P; ke *= P; Kf *= P; Ke *= P; Af *= P; Ae *= P;
+            k0 = mul(k0, P); kf = mul(kf, P); ke = mul(ke, P);
+            Kf = mul(Kf, P); Ke = mul(Ke, P); Af = mul(Af, P); Ae = mul(Ae, P);
+            h = mul(h, P);
         }
-        const R base = drho - R(1.5) * P * uu;
-        Bf = p.wf * base - kf * uu;
+        const R base = mad(h, uu, drho);
+        Bf = mad(p.wf, base, -mul(kf, uu));
 #pragma unroll
-        for (int i = 0; i < 3; ++i) Be[i] = p.we * base + ke * u2[i];
-        eq0 = p.w0 * base + k0 * uu;
+        for (int i = 0; i < 3; ++i) Be[i] = mad(p.we, base, mul(ke, u2[i]));
+        eq0 = mad(p.w0, base, mul(k0, uu));
     }
 
     // Non-equilibrium parts of pair k: s - 2 sym and d - 2 asym, each formed
@@ -498,19 +522,19 @@ struct CellEq {
     __device__ __forceinline__ void neq(R &nsym, R &nasym) const
     {
         constexpr int q = 2 * k + 1;
-        const R cu = R(CX(q)) * u[0] + R(CY(q)) * u[1] + R(CZ(q)) * u[2];
+        const R cu = along(CX(q), CY(q), CZ(q), u);
         R sym, A;
         if (NORM2(q) == 1) {
             const int a = CX(q) ? 0 : (CY(q) ? 1 : 2);
-            sym = Bf + Kf * u2[a];
+            sym = mad(Kf, u2[a], Bf);
             A = Af;
         } else {
             const int c = CX(q) == 0 ? 0 : (CY(q) == 0 ? 1 : 2);
-            sym = Be[c] + Ke * (cu * cu);
+            sym = mad(Ke, mul(cu, cu), Be[c]);
             A = Ae;
         }
-        nsym = fma(R(-2), sym, s[k]);
-        nasym = fma(-A, cu, d[k]);
+        nsym = mad(R(-2), sym, s[k]);
+        nasym = mad(-A, cu, d[k]);
         if constexpr (COMP && !RHO0_IS_RHO && k < 3) nasym -= du[k];
     }
 };
@@ -544,14 +568,13 @@ __device__ __forceinline__ void relax_pair(R g[Q], const CellEq<R, RHO0_IS_RHO, 
     constexpr int q = 2 * k + 1;
     R nsym, nasym;
     e.template neq<k>(nsym, nasym);
-    const R b = fma(p.hm, nasym, -p.force[k]);
+    const R b = mad(p.hm, nasym, -p.force[k]);
     if (ONE_ROUNDING) {
-        g[q] = g[q] - fma(p.hp, nsym, b);
-        g[q + 1] = g[q + 1] - fma(p.hp, nsym, -b);
+        g[q] = g[q] - mad(p.hp, nsym, b);
+        g[q + 1] = g[q + 1] - mad(p.hp, nsym, -b);
     } else {
-        const R a1 = p.hp * nsym;
-        g[q] = (g[q] - a1) - b;
-        g[q + 1] = (g[q + 1] - a1) + b;
+        g[q] = mad(-p.hp, nsym, g[q]) - b;
+        g[q + 1] = mad(-p.hp, nsym, g[q + 1]) + b;
     }
 }
 
@@ -559,7 +582,7 @@ template <typename R, bool RHO0_IS_RHO, bool ONE_ROUNDING>
 __device__ __forceinline__ void collide_lean(R g[Q], const Relax<R> &p)
 {
     const CellEq<R, RHO0_IS_RHO, compensated_v<R, ONE_ROUNDING>> e(g, p);
-    g[0] = fma(-p.wp, g[0] - e.eq0, g[0]);
+    g[0] = mad(-p.wp, g[0] - e.eq0, g[0]);
     relax_pair<R, RHO0_IS_RHO, ONE_ROUNDING, 0>(g, e, p);
     relax_pair<R, RHO0_IS_RHO, ONE_ROUNDING, 1>(g, e, p);
     relax_pair<R, RHO0_IS_RHO, ONE_ROUNDING, 2>(g, e, p);
@@ -597,31 +620,28 @@ __device__ __forceinline__ void collide_mrt(R g[Q], const Relax<R> &p)
     e.template neq<6>(ns[6], na[6]);
     e.template neq<7>(ns[7], na[7]);
     e.template neq<8>(ns[8], na[8]);
-    R faces = R(0), Qn[3] = {R(0), R(0), R(0)};
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int q = 2 * k + 1;
-        if (NORM2(q) == 1) faces += ns[k];
-        else Qn[CX(q) == 0 ? 0 : (CY(q) == 0 ? 1 : 2)] += ns[k];
-    }
+    // pairs 3, 4 are the edges normal to z, 5, 6 to y, 7, 8 to x
+    const R faces = (ns[0] + ns[1]) + ns[2];
+    const R Qn[3] = {ns[7] + ns[8], ns[5] + ns[6], ns[3] + ns[4]};
     const R Qsum = (Qn[0] + Qn[1]) + Qn[2];
-    const R T = fma(R(2), Qsum, faces);
-    const R bT = p.hb * T;       // (omega+ - omega_bulk) T / 2
-    const R bQ = p.h4 * Qsum;    // (omega+ - omega_4) sum Q / 2
-    g[0] = fma(-p.wp, g[0] - e.eq0, g[0]) - R(2) * (bT - bQ);
+    const R T = mad(R(2), Qsum, faces);
+    const R bT = mul(p.hb, T);       // (omega+ - omega_bulk) T / 2
+    const R bQ = mul(p.h4, Qsum);    // (omega+ - omega_4) sum Q / 2
+    const R face0 = mad(bT, third<R>(), -bQ);
+    g[0] = mad(R(-2), bT - bQ, mad(-p.wp, g[0] - e.eq0, g[0]));
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const int q = 2 * k + 1;
         R corr;  // (omega+ - omega_bulk) B / 2 + (omega+ - omega_4) G / 2 for this pair
         if (NORM2(q) == 1) {
             const int a = CX(q) ? 0 : (CY(q) ? 1 : 2);
-            corr = fma(p.h4, Qn[a], bT * R(1.0 / 3.0) - bQ);
+            corr = mad(p.h4, Qn[a], face0);
         } else {
             const int c = CX(q) == 0 ? 0 : (CY(q) == 0 ? 1 : 2);
-            corr = R(0.5) * p.h4 * Qn[c];
+            corr = mul(mul(R(0.5f), p.h4), Qn[c]);
         }
-        const R a1 = fma(p.hp, ns[k], -corr);
-        const R b = fma(p.hm, na[k], -p.force[k]);
+        const R a1 = mad(p.hp, ns[k], -corr);
+        const R b = mad(p.hm, na[k], -p.force[k]);
         if (ONE_ROUNDING) {
             g[q] = g[q] - (a1 + b);
             g[q + 1] = g[q + 1] - (a1 - b);
