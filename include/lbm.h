@@ -105,11 +105,13 @@ typedef struct lbm_ctx *lbm_handle;
 #define LBM_OPT_EQUILIBRIUM 11 /* LBM_EQ_STANDARD or LBM_EQ_IMPROVED */
 #define LBM_OPT_COLLISION 12  /* LBM_SRT, LBM_TRT or LBM_MRT (D3Q19) */
 #define LBM_OPT_BLOCK_X   13  /* step kernel threads per block along x (tuning) */
-#define LBM_OPT_BLOCK_Y   14  /* ... along y; bx * by <= 256 and a multiple of 32 */
+#define LBM_OPT_BLOCK_Y   14  /* ... along y; bx * by <= 256 and a multiple of 32.  The one-cell
+                                 kernels walk the lattice as one sequence of cells in blocks of
+                                 bx * by (if neither was set: of a size the library chooses) */
 #define LBM_OPT_CELLS_X   15  /* cells per thread along x in the step kernel: 1; 2 (paired
                                  accesses; nx even, bx a multiple of 32); or 4 (16-bit storage,
-                                 A/B and AA, nx a multiple of 4, 128-thread blocks shaped from
-                                 nx; otherwise treated as 2).  Default 4 for 16-bit storage, 1
+                                 A/B and AA, nx a multiple of 4; otherwise
+                                 treated as 2).  Default 4 for 16-bit storage, 1
                                  otherwise.  LBM_MRT runs one cell per thread except with 4. */
 #define LBM_OPT_MRT_OMEGA_BULK 16 /* LBM_MRT: rate of the trace of the second-order moments
                                      (bulk viscosity (2/9)(1/omega - 1/2)); 0 < v < 2, default 1 */

@@ -177,13 +177,13 @@ __device__ __forceinline__ void collide27(R g[Q27], const Relax27<R> &p)
 // A/B pull step, one cell per thread.
 template <typename T, bool RHO0, bool WALLS>
 __global__ void __launch_bounds__(256) k27_ab1(const T *__restrict__ src, T *__restrict__ dst, Geo g,
-                                               Relax27<typename Storage<T>::R> p)
+                                               Relax27<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int x, y, z;
+    box.at(i, x, y, z);
     const Site<WALLS> s(x, y, z, 1, g);
     R f[Q27];
 #pragma unroll
@@ -211,16 +211,16 @@ __global__ void __launch_bounds__(256) k27_ab1(const T *__restrict__ src, T *__r
 // A/B pull step for 16-bit storage, four cells per thread (nx % 4 == 0): the
 // same windowed quads as the D3Q19 four-cell step (each +-x shifted window
 // formed by funnel shifts from the aligned quad and its aligned neighbour),
-// 27 populations.  Bitwise the same results as k27_ab1.  ROWS: only the rows
-// y in [r.y0, r.y1), z in [r.z0, r.z0 + gridDim.z) (split_rows).
-template <typename T, bool RHO0, bool WALLS, bool ROWS = false, bool XONLY = false>
+// 27 populations.  Bitwise the same results as k27_ab1.
+template <typename T, bool RHO0, bool WALLS, bool XONLY = false>
 __global__ void __launch_bounds__(128, 4) k27_ab4(const T *__restrict__ src, T *__restrict__ dst, Geo g,
-                                                  Relax27<float> p, Rows r)
+                                                  Relax27<float> p, Box box)
 {
-    const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = (ROWS ? r.y0 : 0) + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = (ROWS ? r.z0 : 0) + (int)blockIdx.z;
-    if (y >= (ROWS ? r.y1 : g.ny) || x0 >= g.nx) return;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int xq, y, z;
+    box.at(i, xq, y, z);
+    const int x0 = 4 * xq;
     Site<WALLS> s(x0, y, z, 4, g);
     drop_yz<XONLY>(s);
     const int xprev = x0 == 0 ? g.nx - 4 : x0 - 4;
@@ -334,16 +334,17 @@ __device__ __forceinline__ void get_canonical(const T *grid, const Site<WALLS> &
 }
 
 #define LBM_Q27_PROLOGUE                                    \
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;    \
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;    \
-    const int z = blockIdx.z;                               \
-    if (x >= g.nx || y >= g.ny) return;                     \
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;    \
+    if (i >= box.count) return;                             \
+    int x, y, z;                                            \
+    box.at(i, x, y, z);                                     \
     const Site<true> s(x, y, z, 1, g);                      \
     const long long cell = s.own + x;
 
 // f = feq(rho, u) (Eq. 14, shifted), written in the A/B layout.
 template <typename T, typename In>
-__global__ void k27_init(T *grid, const In *rho, const In *u, Geo g, Relax27<typename Storage<T>::R> p, int rho0_mode)
+__global__ void k27_init(T *grid, const In *rho, const In *u, Geo g, Relax27<typename Storage<T>::R> p, int rho0_mode,
+                         Box box)
 {
     using R = typename Storage<T>::R;
     LBM_Q27_PROLOGUE
@@ -369,7 +370,7 @@ __global__ void k27_init(T *grid, const In *rho, const In *u, Geo g, Relax27<typ
 
 template <typename T, typename Out>
 __global__ void k27_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, Relax27<typename Storage<T>::R> p,
-                            int rho0_mode)
+                            int rho0_mode, Box box)
 {
     using R = typename Storage<T>::R;
     LBM_Q27_PROLOGUE
@@ -390,7 +391,7 @@ __global__ void k27_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g,
 }
 
 template <typename T>
-__global__ void k27_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g)
+__global__ void k27_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g, Box box)
 {
     LBM_Q27_PROLOGUE
     typename Storage<T>::R fc[Q27];
@@ -400,7 +401,7 @@ __global__ void k27_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g)
 }
 
 template <typename T>
-__global__ void k27_set(T *grid, const T *__restrict__ src, Geo g)
+__global__ void k27_set(T *grid, const T *__restrict__ src, Geo g, Box box)
 {
     LBM_Q27_PROLOGUE
     typename Storage<T>::R fc[Q27];
@@ -425,11 +426,9 @@ static cudaError_t q27_by_prec(int prec, F &&f)
     return cudaErrorInvalidValue;
 }
 
-static dim3 q27_block(const LaunchShape &s) { return dim3(s.bx, s.by, 1); }
-static dim3 q27_grid(const Geo &g, const LaunchShape &s)
-{
-    return dim3((g.nx + s.bx - 1) / s.bx, (g.ny + s.by - 1) / s.by, g.nz);
-}
+constexpr int Q27_THREADS = 256;
+static Box q27_box(const Geo &g) { return Box(g.nx, 0, g.ny, 0, g.nz); }
+static unsigned q27_blocks(const Geo &g) { return blocks_for(g.ncell, Q27_THREADS); }
 
 cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, const CollBoth &c, LaunchShape s,
                           cudaStream_t stream)
@@ -443,52 +442,39 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
         T *b = (T *)dst;
         if constexpr (sizeof(T) == 2) {
             if (s.cells_x == 4 && g.nx % 4 == 0) {
-                // four cells per thread; 128-thread blocks shaped as in the D3Q19 step
-                const int nq = g.nx / 4;
-                int bx = 128, idle = (nq + 127) / 128 * 128 - nq;
-                for (int cw = 64; cw >= 32; cw /= 2) {
-                    const int w = (nq + cw - 1) / cw * cw - nq;
-                    if (w < idle) {
-                        bx = cw;
-                        idle = w;
-                    }
-                }
-                const dim3 bl4(bx, 128 / bx, 1);
-                // with walls, the interior rows run the periodic kernel (or with walls
-                // on x the x-walls-only one) and the wall rows the walled one
-                // (split_rows): walled channel 512x256x256, FP16, 0.68 -> 1.0 of the
-                // copy bandwidth
-                auto run = [&](auto rho0) {
-                    constexpr bool RH = decltype(rho0)::value;
-                    if (!walls) {
-                        const dim3 gr4((g.nx + 4 * bx - 1) / (4 * bx), (g.ny + bl4.y - 1) / bl4.y, g.nz);
-                        q27::k27_ab4<T, RH, false><<<gr4, bl4, 0, stream>>>(a, b, g, p, Rows{0, g.ny, 0});
-                        return;
-                    }
-                    split_rows<true>(g, [&](int kind, Rows r, int nzr) {
-                        const dim3 gr4((g.nx + 4 * bx - 1) / (4 * bx), (r.y1 - r.y0 + bl4.y - 1) / bl4.y, nzr);
+                // four cells per thread; with walls, the interior rows run the periodic
+                // kernel (or with walls on x the x-walls-only one) and the wall rows the
+                // walled one (split_rows): walled channel 512x256x256, FP16, 0.68 -> 1.0
+                // of the copy bandwidth
+                auto run = [&](auto rho0, auto walled) {
+                    constexpr bool RH = decltype(rho0)::value, W = decltype(walled)::value;
+                    split_rows<W>(g, [&](int kind, int y0, int y1, int z0, int planes) {
+                        const Box box(g.nx / 4, y0, y1, z0, planes);
+                        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
                         if (kind == ROWS_WALLED)
-                            q27::k27_ab4<T, RH, true, true><<<gr4, bl4, 0, stream>>>(a, b, g, p, r);
+                            q27::k27_ab4<T, RH, true><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
                         else if (kind == ROWS_XWALLS)
-                            q27::k27_ab4<T, RH, true, true, true><<<gr4, bl4, 0, stream>>>(a, b, g, p, r);
+                            q27::k27_ab4<T, RH, true, true><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
                         else
-                            q27::k27_ab4<T, RH, false, true><<<gr4, bl4, 0, stream>>>(a, b, g, p, r);
+                            q27::k27_ab4<T, RH, false><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
                     });
                 };
-                if (c.rho0_is_rho)
-                    run(std::true_type{});
-                else
-                    run(std::false_type{});
+                if (c.rho0_is_rho && walls) run(std::true_type{}, std::true_type{});
+                else if (c.rho0_is_rho) run(std::true_type{}, std::false_type{});
+                else if (walls) run(std::false_type{}, std::true_type{});
+                else run(std::false_type{}, std::false_type{});
                 return cudaGetLastError();
             }
         }
-        const dim3 gr = q27_grid(g, s), bl = q27_block(s);
+        const int bl = s.threads;
+        const unsigned gr = blocks_for(g.ncell, bl);
+        const Box box = q27_box(g);
         if (c.rho0_is_rho) {
-            if (walls) q27::k27_ab1<T, true, true><<<gr, bl, 0, stream>>>(a, b, g, p);
-            else q27::k27_ab1<T, true, false><<<gr, bl, 0, stream>>>(a, b, g, p);
+            if (walls) q27::k27_ab1<T, true, true><<<gr, bl, 0, stream>>>(a, b, g, p, box);
+            else q27::k27_ab1<T, true, false><<<gr, bl, 0, stream>>>(a, b, g, p, box);
         } else {
-            if (walls) q27::k27_ab1<T, false, true><<<gr, bl, 0, stream>>>(a, b, g, p);
-            else q27::k27_ab1<T, false, false><<<gr, bl, 0, stream>>>(a, b, g, p);
+            if (walls) q27::k27_ab1<T, false, true><<<gr, bl, 0, stream>>>(a, b, g, p, box);
+            else q27::k27_ab1<T, false, false><<<gr, bl, 0, stream>>>(a, b, g, p, box);
         }
         return cudaGetLastError();
     });
@@ -497,19 +483,16 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
 cudaError_t launch_init27(int prec, void *grid, const void *rho, const void *u, int dtype, const Geo &g,
                           const CollBoth &c, cudaStream_t stream)
 {
-    const LaunchShape s{128, 2, 1};
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
         using R = typename Storage<T>::R;
         const q27::Relax27<R> p = q27::to_relax27<R>(c);
         if (dtype == 0)
-            q27::k27_init<T, double><<<q27_grid(g, s), q27_block(s), 0, stream>>>((T *)grid, (const double *)rho,
-                                                                                 (const double *)u, g, p,
-                                                                                 c.rho0_is_rho);
+            q27::k27_init<T, double><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
+                (T *)grid, (const double *)rho, (const double *)u, g, p, c.rho0_is_rho, q27_box(g));
         else
-            q27::k27_init<T, float><<<q27_grid(g, s), q27_block(s), 0, stream>>>((T *)grid, (const float *)rho,
-                                                                                (const float *)u, g, p,
-                                                                                c.rho0_is_rho);
+            q27::k27_init<T, float><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
+                (T *)grid, (const float *)rho, (const float *)u, g, p, c.rho0_is_rho, q27_box(g));
         return cudaGetLastError();
     });
 }
@@ -517,37 +500,34 @@ cudaError_t launch_init27(int prec, void *grid, const void *rho, const void *u, 
 cudaError_t launch_moments27(int prec, const void *grid, void *rho, void *u, int dtype, const Geo &g,
                              const CollBoth &c, cudaStream_t stream)
 {
-    const LaunchShape s{128, 2, 1};
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
         using R = typename Storage<T>::R;
         const q27::Relax27<R> p = q27::to_relax27<R>(c);
         if (dtype == 0)
-            q27::k27_moments<T, double><<<q27_grid(g, s), q27_block(s), 0, stream>>>(
-                (const T *)grid, (double *)rho, (double *)u, g, p, c.rho0_is_rho);
+            q27::k27_moments<T, double><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
+                (const T *)grid, (double *)rho, (double *)u, g, p, c.rho0_is_rho, q27_box(g));
         else
-            q27::k27_moments<T, float><<<q27_grid(g, s), q27_block(s), 0, stream>>>(
-                (const T *)grid, (float *)rho, (float *)u, g, p, c.rho0_is_rho);
+            q27::k27_moments<T, float><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
+                (const T *)grid, (float *)rho, (float *)u, g, p, c.rho0_is_rho, q27_box(g));
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_get27(int prec, const void *grid, void *dst, const Geo &g, cudaStream_t stream)
 {
-    const LaunchShape s{128, 2, 1};
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        q27::k27_get<T><<<q27_grid(g, s), q27_block(s), 0, stream>>>((const T *)grid, (T *)dst, g);
+        q27::k27_get<T><<<q27_blocks(g), Q27_THREADS, 0, stream>>>((const T *)grid, (T *)dst, g, q27_box(g));
         return cudaGetLastError();
     });
 }
 
 cudaError_t launch_set27(int prec, void *grid, const void *src, const Geo &g, cudaStream_t stream)
 {
-    const LaunchShape s{128, 2, 1};
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        q27::k27_set<T><<<q27_grid(g, s), q27_block(s), 0, stream>>>((T *)grid, (const T *)src, g);
+        q27::k27_set<T><<<q27_blocks(g), Q27_THREADS, 0, stream>>>((T *)grid, (const T *)src, g, q27_box(g));
         return cudaGetLastError();
     });
 }

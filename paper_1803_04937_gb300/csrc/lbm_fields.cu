@@ -7,24 +7,22 @@
 
 namespace lbm {
 
-static dim3 cell_block() { return dim3(128, 2, 1); }
-static dim3 cell_grid(const Geo &g)
-{
-    return dim3((g.nx + 127) / 128, (g.ny + 1) / 2, g.nz);
-}
+constexpr int CELL_THREADS = 256;
+static Box cell_box(const Geo &g) { return Box(g.nx, 0, g.ny, 0, g.nz); }
+static unsigned cell_blocks(const Geo &g) { return (unsigned)((g.ncell + CELL_THREADS - 1) / CELL_THREADS); }
 
 #define LBM_CELL_PROLOGUE                                          \
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;           \
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;           \
-    const int z = blockIdx.z;                                      \
-    if (x >= g.nx || y >= g.ny) return;                            \
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;      \
+    if (i >= box.count) return;                                    \
+    int x, y, z;                                                   \
+    box.at(i, x, y, z);                                            \
     Cell c(x, y, z, g);                                            \
-    const long long cell = c.self();
+    const long long cell = i;
 
 // ---------------------------------------------------------------- init
 
 template <typename T, typename In, int D>
-__global__ void k_init(T *grid, const In *rho, const In *u, Geo g, Coll<typename Storage<T>::R> p)
+__global__ void k_init(T *grid, const In *rho, const In *u, Geo g, Coll<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
     LBM_CELL_PROLOGUE
@@ -42,17 +40,18 @@ static cudaError_t init_t(int layout, void *grid, const void *rho, const void *u
     using R = typename Storage<T>::R;
     Coll<R> p = to_coll<R>(cb);
     if (layout == AB)
-        k_init<T, In, D_AB_CANON><<<cell_grid(g), cell_block(), 0, s>>>((T *)grid, (const In *)rho, (const In *)u, g, p);
+        k_init<T, In, D_AB_CANON><<<cell_blocks(g), CELL_THREADS, 0, s>>>((T *)grid, (const In *)rho, (const In *)u, g, p,
+                                                                       cell_box(g));
     else
-        k_init<T, In, D_AB_NEXT><<<cell_grid(g), cell_block(), 0, s>>>((T *)grid, (const In *)rho, (const In *)u,
-                                                                       g, p);  // natural order = AA even layout
+        k_init<T, In, D_AB_NEXT><<<cell_blocks(g), CELL_THREADS, 0, s>>>((T *)grid, (const In *)rho, (const In *)u, g, p,
+                                                                        cell_box(g));  // natural order = AA even layout
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- moments
 
 template <typename T, typename Out, int L>
-__global__ void k_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, Coll<typename Storage<T>::R> p)
+__global__ void k_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, Coll<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
     LBM_CELL_PROLOGUE
@@ -71,7 +70,7 @@ __global__ void k_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, C
 // ---------------------------------------------------------------- canonical copies
 
 template <typename T, int L>
-__global__ void k_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g)
+__global__ void k_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g, Box box)
 {
     LBM_CELL_PROLOGUE
     const int self = (int)cell;
@@ -95,7 +94,7 @@ __global__ void k_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g)
 // CANON_AB = 1: write so that the AB gather returns src; 0: natural order
 // (the AA even layout).
 template <typename T, int CANON_AB>
-__global__ void k_set(T *grid, const T *__restrict__ src, Geo g)
+__global__ void k_set(T *grid, const T *__restrict__ src, Geo g, Box box)
 {
     LBM_CELL_PROLOGUE
     const int self = (int)cell;
@@ -282,14 +281,14 @@ cudaError_t launch_moments(int prec, int layout, const void *grid, void *rho, vo
         const T *gr = (const T *)grid;
         if (dtype == 0) {
             double *r = (double *)rho, *uu = (double *)u;
-            if (layout == AB) k_moments<T, double, AB><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
-            else if (layout == AA_EVEN) k_moments<T, double, AA_EVEN><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
-            else k_moments<T, double, AA_ODD><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
+            if (layout == AB) k_moments<T, double, AB><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
+            else if (layout == AA_EVEN) k_moments<T, double, AA_EVEN><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
+            else k_moments<T, double, AA_ODD><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
         } else {
             float *r = (float *)rho, *uu = (float *)u;
-            if (layout == AB) k_moments<T, float, AB><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
-            else if (layout == AA_EVEN) k_moments<T, float, AA_EVEN><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
-            else k_moments<T, float, AA_ODD><<<cell_grid(g), cell_block(), 0, s>>>(gr, r, uu, g, p);
+            if (layout == AB) k_moments<T, float, AB><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
+            else if (layout == AA_EVEN) k_moments<T, float, AA_EVEN><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
+            else k_moments<T, float, AA_ODD><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
         }
         return cudaGetLastError();
     });
@@ -301,9 +300,9 @@ cudaError_t launch_get_pdfs(int prec, int layout, const void *grid, void *dst, c
         using T = decltype(t);
         const T *gr = (const T *)grid;
         T *d = (T *)dst;
-        if (layout == AB) k_get<T, AB><<<cell_grid(g), cell_block(), 0, s>>>(gr, d, g);
-        else if (layout == AA_EVEN) k_get<T, AA_EVEN><<<cell_grid(g), cell_block(), 0, s>>>(gr, d, g);
-        else k_get<T, AA_ODD><<<cell_grid(g), cell_block(), 0, s>>>(gr, d, g);
+        if (layout == AB) k_get<T, AB><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, d, g, cell_box(g));
+        else if (layout == AA_EVEN) k_get<T, AA_EVEN><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, d, g, cell_box(g));
+        else k_get<T, AA_ODD><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, d, g, cell_box(g));
         return cudaGetLastError();
     });
 }
@@ -314,8 +313,8 @@ cudaError_t launch_set_pdfs(int prec, int layout, void *grid, const void *src, c
         using T = decltype(t);
         T *gr = (T *)grid;
         const T *sr = (const T *)src;
-        if (layout == AB) k_set<T, 1><<<cell_grid(g), cell_block(), 0, s>>>(gr, sr, g);
-        else k_set<T, 0><<<cell_grid(g), cell_block(), 0, s>>>(gr, sr, g);
+        if (layout == AB) k_set<T, 1><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, sr, g, cell_box(g));
+        else k_set<T, 0><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, sr, g, cell_box(g));
         return cudaGetLastError();
     });
 }

@@ -47,14 +47,6 @@ static inline Planes<T> planes_of(void *base, long long ncell)
     return r;
 }
 
-// The rows an A/B launch covers: y in [y0, y1), z in [z0, z0 + gridDim.z).
-// The four-cell step on a lattice with walls on y and/or z runs its interior
-// rows, whose links cross no wall, through the periodic kernel and only the
-// wall rows through the walled one (split_rows).
-struct Rows {
-    int y0, y1, z0;
-};
-
 // Per-thread lattice geometry: wrapped neighbour coordinates, the nine row
 // offsets of the rows y + dy, z + dz (dy, dz in {-1, 0, 1}) and, with walls,
 // the wall flags of the six faces of the cell(s).
@@ -232,13 +224,12 @@ __device__ __forceinline__ void ab1_body(const Planes<T> &src, const Planes<T> &
 
 template <typename T, bool RHO0, bool WALLS, bool MRT = false>
 __global__ void __launch_bounds__(256) k_ab1(Planes<T> src, Planes<T> dst, Geo g, Relax<typename Storage<T>::R> p,
-                                             Rows r)
+                                             Box box)
 {
-    using R = typename Storage<T>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = r.y0 + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = r.z0 + (int)blockIdx.z;
-    if (x >= g.nx || y >= r.y1) return;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int x, y, z;
+    box.at(i, x, y, z);
     if constexpr (WALLS) {
         // warps with no cell at a wall take the periodic body (uniform branch per warp)
         const Site<true> sw(x, y, z, 1, g);
@@ -273,11 +264,8 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(false)) k_aa_even1(Pla
                                                                            Relax<typename Storage<T>::R> p)
 {
     using R = typename Storage<T>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
-    const int own = (z * g.ny + y) * g.nx + x;
+    const unsigned own = blockIdx.x * blockDim.x + threadIdx.x;
+    if (own >= (unsigned)g.ncell) return;
     R f[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) f[q] = Storage<T>::load(P.p[q] + own);
@@ -289,15 +277,15 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(false)) k_aa_even1(Pla
 // AA odd step: read plane qbar at x - c_q, write plane q at x + c_q (through
 // a wall: read plane q / write plane qbar of the own cell).  Every location is
 // read and written by exactly one thread.
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool ROWS = false, bool XONLY = false>
+template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
 __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Planes<T> P, Geo g,
-                                                                         Relax<typename Storage<T>::R> p, Rows r)
+                                                                         Relax<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = (ROWS ? r.y0 : 0) + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = (ROWS ? r.z0 : 0) + (int)blockIdx.z;
-    if (x >= g.nx || y >= (ROWS ? r.y1 : g.ny)) return;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int x, y, z;
+    box.at(i, x, y, z);
     Site<WALLS> s(x, y, z, 1, g);
     drop_yz<XONLY>(s);
     R f[Q];
@@ -621,12 +609,13 @@ constexpr int ab4_blocks = (WALLS && std::is_same_v<T, __half>) ? 4 : 5;
 // little (the end quads' shifted windows take the reflected own quad).
 template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
 __global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Planes<T> src, Planes<T> dst, Geo g,
-                                                                              Relax<float> p, Rows r)
+                                                                              Relax<float> p, Box box)
 {
-    const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = r.y0 + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = r.z0 + (int)blockIdx.z;
-    if (y >= r.y1 || x0 >= g.nx) return;  // no lane needs another lane's data
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;  // no lane needs another lane's data
+    int xq, y, z;
+    box.at(i, xq, y, z);
+    const int x0 = 4 * xq;
     if constexpr (XONLY) {
         Site<true> sx(x0, y, z, 4, g);
         drop_yz<true>(sx);
@@ -654,11 +643,9 @@ __global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Pla
 template <typename T, bool RHO0, bool MRT = false>
 __global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, Geo g, Relax<float> p)
 {
-    const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x0 >= g.nx || y >= g.ny) return;
-    const int own = (z * g.ny + y) * g.nx + x0;
+    const long long first = 4LL * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+    if (first >= g.ncell) return;
+    const int own = (int)first;
     uint2 quad[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q)
@@ -682,19 +669,19 @@ __global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, 
 // quad goes to plane qbar of the own cells.  Each location is written by one
 // thread, and read (for a value that is used) only by that thread, as in the
 // one-cell kernel.
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool ROWS = false, bool XONLY = false>
-__global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g, Relax<float> p, Rows r)
+template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
+__global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g, Relax<float> p, Box box)
 {
     const int lane = threadIdx.x & 31;
-    const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = (ROWS ? r.y0 : 0) + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-    const int z = (ROWS ? r.z0 : 0) + (int)blockIdx.z;
-    if (y >= (ROWS ? r.y1 : g.ny)) return;  // uniform across the warp
-    const bool active = x0 < g.nx;
-    Site<WALLS> s(active ? x0 : 0, y, z, 4, g);
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool active = i < box.count;
+    int xq, y, z;
+    box.at(active ? i : box.count - 1u, xq, y, z);
+    Site<WALLS> s(4 * xq, y, z, 4, g);
     drop_yz<XONLY>(s);
-    const int xs = s.x;
-    const bool last = lane == 31 || xs + 4 >= g.nx;
+    // ends of the lanes' segment of a row (a warp may hold several rows' ends)
+    const bool head = lane == 0 || xq == 0;
+    const bool last = lane == 31 || s.x + 4 >= g.nx || i + 1 >= box.count;
     uint2 quad[Q];
     load4w<true>(P, s, g, quad);
     if (active) collide4<T, RHO0, MRT>(quad, p);
@@ -718,7 +705,7 @@ __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g
                 continue;
             }
             unsigned short *t = dst + trow + sw.x;
-            if (lane == 0) {  // element x0 belongs to the previous segment's last cell
+            if (head) {  // element x0 belongs to the previous segment's last cell
                 t[1] = (unsigned short)(quad[q].x & 0xffffu);
                 *reinterpret_cast<unsigned int *>(t + 2) = __byte_perm(quad[q].x, quad[q].y, 0x5432);
             } else {
@@ -747,7 +734,7 @@ __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g
                 v.y = __byte_perm(quad[q].y, rgt, 0x5432);
                 *reinterpret_cast<uint2 *>(t) = v;
             }
-            if (lane == 0)  // cell x0 goes to x0 - 1: the previous segment, the periodic image, or a wall
+            if (head)  // cell x0 goes to x0 - 1: the previous segment, the periodic image, or a wall
                 *((WALLS && s.bxm) ? bnc + sw.own + sw.x : dst + trow + sw.xm) = (unsigned short)(quad[q].x & 0xffffu);
         }
     }
@@ -770,68 +757,74 @@ __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g
 // Kinds of the launches of split_rows.
 enum { ROWS_PERIODIC = 0, ROWS_WALLED = 1, ROWS_XWALLS = 2 };
 
+// launch(kind, y0, y1, z0, planes)
 template <bool WALLS, typename F>
 static void split_rows(const Geo &g, F &&launch)
 {
     if (!WALLS) {
-        launch(ROWS_PERIODIC, Rows{0, g.ny, 0}, g.nz);
+        launch(ROWS_PERIODIC, 0, g.ny, 0, g.nz);
         return;
     }
     const int inner = g.wall_x ? ROWS_XWALLS : ROWS_PERIODIC;
     const int ylo = g.wall_y ? 1 : 0, yhi = g.wall_y ? g.ny - 1 : g.ny;
     const int zlo = g.wall_z ? 1 : 0, zhi = g.wall_z ? g.nz - 1 : g.nz;
-    if (yhi > ylo && zhi > zlo) launch(inner, Rows{ylo, yhi, zlo}, zhi - zlo);
+    if (yhi > ylo && zhi > zlo) launch(inner, ylo, yhi, zlo, zhi - zlo);
     if (g.wall_y) {
-        launch(ROWS_WALLED, Rows{0, 1, 0}, g.nz);
-        if (g.ny > 1) launch(ROWS_WALLED, Rows{g.ny - 1, g.ny, 0}, g.nz);
+        launch(ROWS_WALLED, 0, 1, 0, g.nz);
+        if (g.ny > 1) launch(ROWS_WALLED, g.ny - 1, g.ny, 0, g.nz);
     }
     if (g.wall_z && yhi > ylo) {
-        launch(ROWS_WALLED, Rows{ylo, yhi, 0}, 1);
-        if (g.nz > 1) launch(ROWS_WALLED, Rows{ylo, yhi, g.nz - 1}, 1);
+        launch(ROWS_WALLED, ylo, yhi, 0, 1);
+        if (g.nz > 1) launch(ROWS_WALLED, ylo, yhi, g.nz - 1, 1);
     }
 }
+
+static inline unsigned blocks_for(long long items, int threads) { return (unsigned)((items + threads - 1) / threads); }
 
 // The one-cell A/B step stays one launch over all rows: its walled kernel
 // already runs at the periodic kernel's speed (walled channel 512x256x256,
 // FP32: 45.2 GLUPS as one launch, 44.8 split).
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_ab1(const Planes<T> &S, const Planes<T> &D, const Geo &g, const Relax<typename Storage<T>::R> &p,
-                       dim3 block, cudaStream_t stream)
+                       int threads, cudaStream_t stream)
 {
-    const dim3 grid((g.nx + block.x - 1) / block.x, (g.ny + block.y - 1) / block.y, g.nz);
-    k_ab1<T, RHO0, WALLS, MRT><<<grid, block, 0, stream>>>(S, D, g, p, Rows{0, g.ny, 0});
+    const Box box(g.nx, 0, g.ny, 0, g.nz);
+    k_ab1<T, RHO0, WALLS, MRT><<<blocks_for(box.count, threads), threads, 0, stream>>>(S, D, g, p, box);
 }
 
 // The one-cell AA odd step, split into interior and wall rows like the
 // four-cell one (walled channel 512x256x256, FP32: odd step 0.72 of the copy
 // bandwidth as one walled launch).
 template <typename T, bool RHO0, bool WALLS, bool MRT>
-static void launch_aa_odd1(const Planes<T> &P, const Geo &g, const Relax<typename Storage<T>::R> &p, dim3 block,
+static void launch_aa_odd1(const Planes<T> &P, const Geo &g, const Relax<typename Storage<T>::R> &p, int threads,
                            cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, Rows r, int nzr) {
-        const dim3 grid((g.nx + block.x - 1) / block.x, (r.y1 - r.y0 + block.y - 1) / block.y, nzr);
+    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
+        const Box box(g.nx, y0, y1, z0, planes);
+        const unsigned grid = blocks_for(box.count, threads);
         if (kind == ROWS_WALLED)
-            k_aa_odd1<T, RHO0, true, MRT, WALLS><<<grid, block, 0, stream>>>(P, g, p, r);
+            k_aa_odd1<T, RHO0, true, MRT><<<grid, threads, 0, stream>>>(P, g, p, box);
         else if (kind == ROWS_XWALLS)
-            k_aa_odd1<T, RHO0, true, MRT, true, true><<<grid, block, 0, stream>>>(P, g, p, r);
+            k_aa_odd1<T, RHO0, true, MRT, true><<<grid, threads, 0, stream>>>(P, g, p, box);
         else
-            k_aa_odd1<T, RHO0, false, MRT, WALLS><<<grid, block, 0, stream>>>(P, g, p, r);
+            k_aa_odd1<T, RHO0, false, MRT><<<grid, threads, 0, stream>>>(P, g, p, box);
     });
 }
 
+constexpr int QUAD_THREADS = 128;  // threads per block of the four-cell kernels
+
 template <typename T, bool RHO0, bool WALLS, bool MRT>
-static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, const Relax<float> &p, dim3 block4,
-                       cudaStream_t stream)
+static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, Rows r, int nzr) {
-        const dim3 grid((g.nx + 4 * block4.x - 1) / (4 * block4.x), (r.y1 - r.y0 + block4.y - 1) / block4.y, nzr);
+    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
+        const Box box(g.nx / 4, y0, y1, z0, planes);
+        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
         if (kind == ROWS_WALLED)
-            k_ab4<T, RHO0, true, MRT><<<grid, block4, 0, stream>>>(S, D, g, p, r);
+            k_ab4<T, RHO0, true, MRT><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
         else if (kind == ROWS_XWALLS)
-            k_ab4<T, RHO0, true, MRT, true><<<grid, block4, 0, stream>>>(S, D, g, p, r);
+            k_ab4<T, RHO0, true, MRT, true><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
         else
-            k_ab4<T, RHO0, false, MRT><<<grid, block4, 0, stream>>>(S, D, g, p, r);
+            k_ab4<T, RHO0, false, MRT><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
     });
 }
 
@@ -841,21 +834,48 @@ static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, con
 // launch.  Each location is read and written by one cell's thread only, so
 // the launches may run in any order.
 template <typename T, bool RHO0, bool WALLS, bool MRT>
-static void launch_aa_odd4(const Planes<T> &P, const Geo &g, const Relax<float> &p, dim3 block4, cudaStream_t stream)
+static void launch_aa_odd4(const Planes<T> &P, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, Rows r, int nzr) {
-        const dim3 grid((g.nx + 4 * block4.x - 1) / (4 * block4.x), (r.y1 - r.y0 + block4.y - 1) / block4.y, nzr);
+    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
+        const Box box(g.nx / 4, y0, y1, z0, planes);
+        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
         // the interior rows of a walled lattice take the x-walls-only kernel also
         // without x walls (its x flags are then false): it compiles to a faster
         // step than the periodic kernel with a row range (walled channel, FP16 AA
         // pair 0.81 -> 0.85, BF16 0.80 -> 0.82)
         if (kind == ROWS_WALLED)
-            k_aa_odd4<T, RHO0, true, MRT, WALLS><<<grid, block4, 0, stream>>>(P, g, p, r);
+            k_aa_odd4<T, RHO0, true, MRT><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
         else if (WALLS)
-            k_aa_odd4<T, RHO0, true, MRT, true, true><<<grid, block4, 0, stream>>>(P, g, p, r);
+            k_aa_odd4<T, RHO0, true, MRT, true><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
         else
-            k_aa_odd4<T, RHO0, false, MRT><<<grid, block4, 0, stream>>>(P, g, p, r);
+            k_aa_odd4<T, RHO0, false, MRT><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
     });
+}
+
+// One-cell step of either pattern.
+template <typename T, bool RHO0, bool WALLS, bool MRT>
+static void launch_step1(int kind, void *src, const Planes<T> &D, const Geo &g,
+                         const Relax<typename Storage<T>::R> &p, int threads, cudaStream_t stream)
+{
+    if (kind == 0)
+        launch_ab1<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, threads, stream);
+    else if (kind == 1)
+        k_aa_even1<T, RHO0, MRT><<<blocks_for(g.ncell, threads), threads, 0, stream>>>(D, D, g, p);
+    else
+        launch_aa_odd1<T, RHO0, WALLS, MRT>(D, g, p, threads, stream);
+}
+
+// Four-cell step of either pattern (16-bit storage, nx a multiple of 4).
+template <typename T, bool RHO0, bool WALLS, bool MRT>
+static void launch_step4(int kind, void *src, const Planes<T> &D, const Geo &g, const Relax<float> &p,
+                         cudaStream_t stream)
+{
+    if (kind == 0)
+        launch_ab4<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, stream);
+    else if (kind == 1)
+        k_aa_even4<T, RHO0, MRT><<<blocks_for(g.ncell / 4, QUAD_THREADS), QUAD_THREADS, 0, stream>>>(D, D, g, p);
+    else
+        launch_aa_odd4<T, RHO0, WALLS, MRT>(D, g, p, stream);
 }
 
 template <typename T, bool RHO0, bool WALLS>
@@ -864,76 +884,32 @@ static cudaError_t step_t(int kind, void *src, void *dst, const Geo &g, const Co
 {
     using R = typename Storage<T>::R;
     const Relax<R> p = to_relax<R>(cb);
-    const dim3 block(ls.bx, ls.by, 1);
-    const bool quads = sizeof(T) == 2 && ls.cells_x == 4 && (g.nx % 4) == 0;
-    if (cb.mrt && !quads) {
-        // MRT: one cell per thread (16-bit storage with nx % 4 == 0 takes the four-cell kernels below)
-        const dim3 grid1((g.nx + ls.bx - 1) / ls.bx, (g.ny + ls.by - 1) / ls.by, g.nz);
-        const Planes<T> D = planes_of<T>(dst, g.ncell);
-        if (kind == 0)
-            launch_ab1<T, RHO0, WALLS, true>(planes_of<T>(src, g.ncell), D, g, p, block, stream);
-        else if (kind == 1)
-            k_aa_even1<T, RHO0, true><<<grid1, block, 0, stream>>>(D, D, g, p);
-        else
-            launch_aa_odd1<T, RHO0, WALLS, true>(D, g, p, block, stream);
-        return cudaGetLastError();
-    }
-    const bool pairs = !quads && ls.cells_x >= 2 && (g.nx % 2) == 0 && (ls.bx % 32) == 0;
-    if (quads) {
-        // 128 threads; bx in {128, 64, 32} along x (whole warps per row segment), the
-        // rest along y; bx leaves the fewest idle lanes at the end of a row (nx = 768:
-        // 64, so three blocks cover the 192 quads of a row instead of two with 64
-        // idle lanes), the larger on ties
-        const int nq = g.nx / 4;
-        int bx = 128, idle = (nq + 127) / 128 * 128 - nq;
-        for (int c = 64; c >= 32; c /= 2) {
-            const int w = (nq + c - 1) / c * c - nq;
-            if (w < idle) {
-                bx = c;
-                idle = w;
-            }
-        }
-        const dim3 block4(bx, 128 / bx, 1);
-        const dim3 grid4((g.nx + 4 * bx - 1) / (4 * bx), (g.ny + block4.y - 1) / block4.y, g.nz);
-        if constexpr (sizeof(T) == 2) {
-            const Planes<T> D = planes_of<T>(dst, g.ncell);
-            if (cb.mrt) {
-                if (kind == 0)
-                    launch_ab4<T, RHO0, WALLS, true>(planes_of<T>(src, g.ncell), D, g, p, block4, stream);
-                else if (kind == 1)
-                    k_aa_even4<T, RHO0, true><<<grid4, block4, 0, stream>>>(D, D, g, p);
-                else
-                    launch_aa_odd4<T, RHO0, WALLS, true>(D, g, p, block4, stream);
-            } else if (kind == 0) {
-                launch_ab4<T, RHO0, WALLS, false>(planes_of<T>(src, g.ncell), D, g, p, block4, stream);
-            } else if (kind == 1) {
-                k_aa_even4<T, RHO0><<<grid4, block4, 0, stream>>>(D, D, g, p);
-            } else {
-                launch_aa_odd4<T, RHO0, WALLS, false>(D, g, p, block4, stream);
-            }
-        }
-        return cudaGetLastError();
-    }
-    const int span = pairs ? 2 * ls.bx : ls.bx;
-    const dim3 grid((g.nx + span - 1) / span, (g.ny + ls.by - 1) / ls.by, g.nz);
     const Planes<T> D = planes_of<T>(dst, g.ncell);
-    if (kind == 0) {
-        const Planes<T> S = planes_of<T>(src, g.ncell);
-        if (pairs)
-            k_ab2<T, RHO0, WALLS><<<grid, block, 0, stream>>>(S, D, g, p);
-        else
-            launch_ab1<T, RHO0, WALLS, false>(S, D, g, p, block, stream);
-    } else if (kind == 1) {
-        if (pairs)
+    const int threads = ls.threads;
+    if constexpr (sizeof(T) == 2) {
+        if (ls.cells_x == 4 && g.nx % 4 == 0) {
+            if (cb.mrt)
+                launch_step4<T, RHO0, WALLS, true>(kind, src, D, g, p, stream);
+            else
+                launch_step4<T, RHO0, WALLS, false>(kind, src, D, g, p, stream);
+            return cudaGetLastError();
+        }
+    }
+    if (!cb.mrt && ls.cells_x >= 2 && (g.nx % 2) == 0 && (ls.bx % 32) == 0) {
+        const dim3 block(ls.bx, ls.by, 1);
+        const dim3 grid((g.nx + 2 * ls.bx - 1) / (2 * ls.bx), (g.ny + ls.by - 1) / ls.by, g.nz);
+        if (kind == 0)
+            k_ab2<T, RHO0, WALLS><<<grid, block, 0, stream>>>(planes_of<T>(src, g.ncell), D, g, p);
+        else if (kind == 1)
             k_aa_even2<T, RHO0><<<grid, block, 0, stream>>>(D, g, p);
         else
-            k_aa_even1<T, RHO0><<<grid, block, 0, stream>>>(D, D, g, p);
-    } else {
-        if (pairs)
             k_aa_odd2<T, RHO0, WALLS><<<grid, block, 0, stream>>>(D, g, p);
-        else
-            launch_aa_odd1<T, RHO0, WALLS, false>(D, g, p, block, stream);
+        return cudaGetLastError();
     }
+    if (cb.mrt)
+        launch_step1<T, RHO0, WALLS, true>(kind, src, D, g, p, threads, stream);
+    else
+        launch_step1<T, RHO0, WALLS, false>(kind, src, D, g, p, threads, stream);
     return cudaGetLastError();
 }
 
