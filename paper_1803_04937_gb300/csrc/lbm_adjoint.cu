@@ -127,34 +127,6 @@ __device__ __forceinline__ void adj_pair(const CellEq<R, false> &e, const R mu[Q
     cf += D * fraw[k];
 }
 
-// Double-float numbers: an unevaluated sum hi + lo of two floats.  Sums of
-// FP32 terms built with error-free transformations (TwoSum) keep about 48
-// bits, as many as FP64 sums of the same FP32 terms would, and run on the FP32
-// pipe.
-struct DF {
-    float hi, lo;
-};
-
-__device__ __forceinline__ DF df_add(DF a, DF b)
-{
-    const float s = a.hi + b.hi;
-    const float bv = s - a.hi;
-    float e = (a.hi - (s - bv)) + (b.hi - bv);
-    e += a.lo + b.lo;
-    const float hi = s + e;
-    return DF{hi, e - (hi - s)};
-}
-
-__device__ __forceinline__ DF df_warp_sum(DF a)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const DF b{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};
-        a = df_add(a, b);
-    }
-    return a;
-}
-
 // The adjoint of one cell: from the forward populations f of the state at t
 // (rho0 = 1) and mu = S^T lambda(t+1), the cell's lambda(t) (out) and its
 // terms of dL/domega+ (gp) and dL/domega- (gm).

@@ -183,27 +183,6 @@ struct Cell {
 //             number of AA steps).
 enum Layout { AB = 0, AA_EVEN = 1, AA_ODD = 2 };
 
-template <int L, typename T, typename R>
-__device__ __forceinline__ void gather(const T *grid, const Cell &c, long long ncell, R g[Q])
-{
-    const int self = c.self();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        long long off;
-        if (L == AA_EVEN) {
-            off = (long long)q * ncell + self;
-        } else {
-            bool wall;
-            int src = c.template along<-1>(q, wall);
-            if (L == AB)
-                off = wall ? (long long)OPP(q) * ncell + self : (long long)q * ncell + src;
-            else
-                off = wall ? (long long)q * ncell + self : (long long)OPP(q) * ncell + src;
-        }
-        g[q] = Storage<T>::load(grid + off);
-    }
-}
-
 // Where post-collision values of a step go:
 //   AB_NEXT : grid[q][x]                 (pull scheme, next step gathers them)
 //   AA_EVEN : grid[qbar][x]
@@ -254,24 +233,6 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
         v = lane < nw ? sh[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    }
-    return v;
-}
-
-__device__ __forceinline__ double block_max(double v, double *sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    v = 0.0;
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        v = lane < nw ? sh[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
     }
     return v;
 }
@@ -467,6 +428,34 @@ __device__ __forceinline__ void two_sum_acc(R &hi, R &lo, R v)
     const R bv = s - hi;
     lo += (hi - (s - bv)) + (v - bv);
     hi = s;
+}
+
+// Double-float numbers: an unevaluated sum hi + lo of two floats.  Sums of
+// FP32 terms built with error-free transformations (TwoSum) keep about 48
+// bits, as many as FP64 sums of the same FP32 terms would, and run on the FP32
+// pipe.
+struct DF {
+    float hi, lo;
+};
+
+__device__ __forceinline__ DF df_add(DF a, DF b)
+{
+    const float s = a.hi + b.hi;
+    const float bv = s - a.hi;
+    float e = (a.hi - (s - bv)) + (b.hi - bv);
+    e += a.lo + b.lo;
+    const float hi = s + e;
+    return DF{hi, e - (hi - s)};
+}
+
+__device__ __forceinline__ DF df_warp_sum(DF a)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const DF b{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};
+        a = df_add(a, b);
+    }
+    return a;
 }
 
 // c_q . u of a lattice direction (c: its components, -1, 0 or 1) without the

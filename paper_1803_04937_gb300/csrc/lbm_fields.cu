@@ -4,6 +4,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
+#include "lbm_step.cuh"  // Planes, Site, gather1
 
 namespace lbm {
 
@@ -18,6 +19,37 @@ static unsigned cell_blocks(const Geo &g) { return (unsigned)((g.ncell + CELL_TH
     box.at(i, x, y, z);                                            \
     Cell c(x, y, z, g);                                            \
     const long long cell = i;
+
+// The populations f_q - w_q of one cell in layout L, with the step kernels'
+// addressing (plane pointers from the parameters, 32-bit offsets, no wall logic
+// on periodic lattices).
+template <int L, bool WALLS, typename T, typename R>
+__device__ __forceinline__ void gather_state(const Planes<T> &P, const Site<WALLS> &s, R f[Q])
+{
+    if constexpr (L == AA_EVEN) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f[q] = Storage<T>::load(P.p[q] + s.own + s.x);
+    } else {
+        gather1<L == AA_ODD>(P, s, f);
+    }
+}
+
+// Calls f(layout, walls) with both as compile-time constants (an AA even state
+// needs no neighbours, so no walls either).
+template <typename F>
+static cudaError_t by_layout(int layout, const Geo &g, F &&f)
+{
+    using LAB = std::integral_constant<int, AB>;
+    using LEven = std::integral_constant<int, AA_EVEN>;
+    using LOdd = std::integral_constant<int, AA_ODD>;
+    const bool walls = g.wall_x || g.wall_y || g.wall_z;
+    if (layout == AA_EVEN) f(LEven{}, std::false_type{});
+    else if (layout == AB && walls) f(LAB{}, std::true_type{});
+    else if (layout == AB) f(LAB{}, std::false_type{});
+    else if (walls) f(LOdd{}, std::true_type{});
+    else f(LOdd{}, std::false_type{});
+    return cudaGetLastError();
+}
 
 // ---------------------------------------------------------------- init
 
@@ -50,15 +82,20 @@ static cudaError_t init_t(int layout, void *grid, const void *rho, const void *u
 
 // ---------------------------------------------------------------- moments
 
-template <typename T, typename Out, int L>
-__global__ void k_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, Coll<typename Storage<T>::R> p, Box box)
+template <typename T, typename Out, int L, bool WALLS>
+__global__ void __launch_bounds__(CELL_THREADS) k_moments(Planes<T> P, Out *rho, Out *u, Geo g,
+                                                          Coll<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    LBM_CELL_PROLOGUE
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int x, y, z;
+    box.at(i, x, y, z);
     R f[Q];
-    gather<L>(grid, c, g.ncell, f);
+    gather_state<L>(P, Site<WALLS>(x, y, z, 1, g), f);
     R drho, rho0, uv[3];
     macro(f, p, drho, rho0, uv);
+    const long long cell = i;
     if (rho) rho[cell] = Out(R(1) + drho);
     if (u) {
         u[cell] = Out(uv[0]);
@@ -115,126 +152,276 @@ __global__ void k_set(T *grid, const T *__restrict__ src, Geo g, Box box)
 // ---------------------------------------------------------------- reductions
 
 constexpr int RED_THREADS = 256;
-constexpr int RED_BLOCKS = 152 * 4;
+constexpr int RED_SMS = 152, RED_BLOCKS = RED_SMS * 4;  // all resident at once
 int reduce_blocks() { return RED_BLOCKS; }
 
-template <typename T, int L>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce(const T *__restrict__ grid, double *partial, Geo g,
-                                                        Coll<typename Storage<T>::R> p)
+// A running sum.  This GPU adds about 64 FP32 numbers in the time of one FP64
+// number, so cells of FP32 arithmetic are summed in double-float (TwoSum; exact
+// products by fma), which keeps more bits of such terms than they have, and the
+// few cells' sum is added to an FP64 total before its own rounding matters.
+template <typename R> struct Sum;
+template <> struct Sum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) { two_sum_acc(hi, lo, v); }
+    __device__ __forceinline__ void add_product(float a, float b)
+    {
+        const float p = __fmul_rn(a, b);
+        two_sum_acc(hi, lo, p);
+        lo += fmaf(a, b, -p);
+    }
+    __device__ __forceinline__ void flush(double &total)
+    {
+        total += (double)hi + (double)lo;
+        hi = lo = 0.f;
+    }
+};
+template <> struct Sum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add_product(double a, double b) { v = fma(a, b, v); }
+    __device__ __forceinline__ void flush(double &total)
+    {
+        total += v;
+        v = 0.0;
+    }
+};
+constexpr int SUM_CELLS = 16;  // cells between two flushes
+
+// Whether products of FP32 numbers whose largest square is about v can be split
+// into value and rounding error in FP32: not where they come near its range's
+// ends (nor for NaN); those few cells are summed in FP64 at once.
+__device__ __forceinline__ bool fits_products(float v) { return v > 1e-20f && v < 1e30f; }
+__device__ __forceinline__ bool fits_products(double v) { return isfinite(v); }
+
+__device__ __forceinline__ double warp_sum_or_max(double v, bool largest)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double w = __shfl_down_sync(0xffffffffu, v, o);
+        v = largest ? fmax(v, w) : v + w;
+    }
+    return v;
+}
+
+// Mass, energy, momentum, max |u| and non-finite cells: one partial row per
+// block of a fixed grid, in a fixed order (deterministic for a lattice size).
+// The kernel was bound by FP64 work, about 45 operations a cell (a square root
+// among them) and a 64-bit division; with the sums above, the root taken of the
+// thread's largest |u|^2 only and the row found by a multiplication it is bound
+// by its loads.
+template <typename T, int L, bool WALLS>
+__global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
+    k_reduce(Planes<T> P, double *partial, Geo g, Coll<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    __shared__ double sh[32];
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    const long long nxy = (long long)g.nx * g.ny;
+    __shared__ double sh[7][RED_THREADS];
+    double acc[5] = {0, 0, 0, 0, 0}, uumax = 0.0;  // drho, |u|^2, rho0 u; largest |u|^2
+    Sum<R> sum[5];
+    R near_max = R(-1);  // |u|^2 below this cannot be the largest
+    int bad = 0, n = 0;
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncell;
          cell += (long long)gridDim.x * blockDim.x) {
-        const int z = (int)(cell / nxy);
-        const int rem = (int)(cell - z * nxy);
-        const int y = rem / g.nx;
-        const int x = rem - y * g.nx;
-        Cell c(x, y, z, g);
+        int x, y, z;
+        box.at((unsigned)cell, x, y, z);
         R f[Q];
-        gather<L>(grid, c, g.ncell, f);
-        bool bad = false;
+        gather_state<L>(P, Site<WALLS>(x, y, z, 1, g), f);
+        R drho, rho0, u[3];
+        macro(f, p, drho, rho0, u);
+        bool finite = isfinite(drho);  // a sum with an infinity or a NaN in it is not finite
+        if (!finite) {
+            finite = true;
 #pragma unroll
-        for (int q = 0; q < Q; ++q) bad |= !isfinite(f[q]);
-        R drho, rho0, uv[3];
-        macro(f, p, drho, rho0, uv);
-        double u0 = uv[0], u1 = uv[1], u2 = uv[2];
-        double r0 = rho0;
-        double uu = u0 * u0 + u1 * u1 + u2 * u2;
-        acc[0] += (double)drho;
-        acc[1] += 0.5 * uu;
-        acc[2] += r0 * u0 - (double)p.half_a[0];
-        acc[3] += r0 * u1 - (double)p.half_a[1];
-        acc[4] += r0 * u2 - (double)p.half_a[2];
-        acc[5] = fmax(acc[5], sqrt(uu));
-        acc[6] += bad ? 1.0 : 0.0;
+            for (int q = 0; q < Q; ++q) finite &= isfinite(f[q]);
+        }
+        const R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        bad += !finite;
+        if (finite && fits_products(uu) && isfinite(drho)) {
+            sum[0].add(drho);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                sum[1].add_product(u[i], u[i]);
+                if (p.rho0_is_rho)
+                    sum[2 + i].add_product(rho0, u[i]);
+                else
+                    sum[2 + i].add(u[i]);
+            }
+        } else {
+            acc[0] += (double)drho;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                acc[1] += (double)u[i] * (double)u[i];
+                acc[2 + i] += (double)rho0 * (double)u[i];
+            }
+        }
+        if (!(uu < near_max)) {
+            const double v[3] = {(double)u[0], (double)u[1], (double)u[2]};
+            uumax = fmax(uumax, v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+            near_max = R(uumax) * R(0.999999);
+        }
+        if (++n % SUM_CELLS == 0) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
+        }
     }
 #pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        double v = (k == 5) ? block_max(acc[k], sh) : block_sum(acc[k], sh);
-        if (threadIdx.x == 0) partial[blockIdx.x * 8 + k] = v;
+    for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
+    acc[1] *= 0.5;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) acc[2 + i] -= n * (double)p.half_a[i];  // rho0 u = j + a/2
+    // one warp per result sums the block's threads (a shuffle tree of every warp
+    // for every result would cost four times the FP64 additions)
+    const double slot[7] = {acc[0], acc[1], acc[2], acc[3], acc[4], sqrt(uumax), (double)bad};
+#pragma unroll
+    for (int k = 0; k < 7; ++k) sh[k][threadIdx.x] = slot[k];
+    __syncthreads();
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k < 7) {
+        double v = sh[k][lane];
+#pragma unroll
+        for (int i = 32; i < RED_THREADS; i += 32) v = (k == 5) ? fmax(v, sh[k][lane + i]) : v + sh[k][lane + i];
+        v = warp_sum_or_max(v, k == 5);
+        if (lane == 0) partial[blockIdx.x * 8 + k] = v;
     }
 }
 
+// One warp per result, so that all rows' loads are in flight together.
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *partial, int nblocks, double *result,
                                                               double ncell)
 {
-    __shared__ double sh[32];
-    for (int k = 0; k < 7; ++k) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-            v = (k == 5) ? fmax(v, partial[b * 8 + k]) : v + partial[b * 8 + k];
-        v = (k == 5) ? block_max(v, sh) : block_sum(v, sh);
-        if (threadIdx.x == 0) result[k] = (k == 0) ? ncell + v : v;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v = 0.0;
+    if (k < 7) {
+        constexpr int U = 20;  // loads in flight
+        for (int b = lane; b < nblocks; b += 32 * U) {
+            double row[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) row[i] = b + 32 * i < nblocks ? partial[(b + 32 * i) * 8 + k] : 0.0;
+#pragma unroll
+            for (int i = 0; i < U; ++i) v = (k == 5) ? fmax(v, row[i]) : v + row[i];
+        }
+        v = warp_sum_or_max(v, k == 5);
     }
-    if (threadIdx.x == 0) result[7] = 0.0;
+    if (lane == 0) result[k] = (k == 0) ? ncell + v : v;  // slot 7 is 0
 }
 
 // Enstrophy 1/2 <|curl u|^2> of the state, with second-order central
 // differences of u (Eq. 17) between the axis neighbours.  Periodic axes wrap;
 // across a half-way bounce-back wall the ghost velocity is -u of the own cell
-// (the wall at rest halfway between them).  Each cell gathers its six
-// neighbours' populations (off the per-step path; the neighbours' rows are
-// shared through L1/L2).  Deterministic: fixed grid, fixed per-thread order,
-// fixed trees.
-template <typename T, int L>
-__device__ __forceinline__ void velocity_at(const T *__restrict__ grid, int x, int y, int z, const Geo &g,
-                                            const Coll<typename Storage<T>::R> &p, double u[3])
+// (the wall at rest halfway between them).  A block owns a tile of ENS_X x
+// ENS_Y columns with a halo of one and marches along z: every thread forms the
+// velocity of its column's cell once per plane, keeps those of three planes in
+// registers and shares the middle one through shared memory.  (Gathering all
+// six neighbours' populations instead took 133 loads a cell and FP64
+// differences: 192^3 FP16 1.2 ms.)  Differences of FP32 velocities are taken
+// exactly in double-float, FP64 storage uses FP64.  Deterministic: fixed grid,
+// fixed tiles, fixed per-thread order, fixed trees.
+constexpr int ENS_LANES = 32, ENS_ROWS = 16, ENS_THREADS = ENS_LANES * ENS_ROWS;
+constexpr int ENS_X = ENS_LANES - 2, ENS_Y = ENS_ROWS - 2;
+constexpr int ENS_PER_SM = 2;  // resident blocks
+
+// Planes per tile: the resident blocks take the tiles in turns, and each tile
+// costs two more planes than it has.
+static int enstrophy_planes(const Geo &g)
 {
-    using R = typename Storage<T>::R;
-    const Cell c(x, y, z, g);
-    R f[Q];
-    gather<L>(grid, c, g.ncell, f);
-    R drho, rho0, uv[3];
-    macro(f, p, drho, rho0, uv);
-    u[0] = uv[0];
-    u[1] = uv[1];
-    u[2] = uv[2];
+    const long long columns = (long long)((g.nx + ENS_X - 1) / ENS_X) * ((g.ny + ENS_Y - 1) / ENS_Y);
+    long long best = -1;
+    int planes = g.nz;
+    for (int len = 1; len <= g.nz; len += 1 + len / 16) {
+        const long long tiles = columns * ((g.nz + len - 1) / len);
+        const long long cost = (tiles + RED_SMS * ENS_PER_SM - 1) / (RED_SMS * ENS_PER_SM) * (len + 2);
+        if (best < 0 || cost < best) {
+            best = cost;
+            planes = len;
+        }
+    }
+    return planes;
 }
 
-template <typename T, int L>
-__global__ void __launch_bounds__(RED_THREADS) k_enstrophy(const T *__restrict__ grid, double *partial, Geo g,
-                                                           Coll<typename Storage<T>::R> p)
+// a - b, exact as a double-float
+__device__ __forceinline__ DF exact_diff(float a, float b)
 {
+    DF r{a, 0.f};
+    two_sum_acc(r.hi, r.lo, -b);
+    return r;
+}
+// (a1 - a0) - (b1 - b0), twice a component of the curl, squared and added to s or total
+__device__ __forceinline__ void add_square_of_curl(Sum<float> &s, double &total, float a1, float a0, float b1, float b0)
+{
+    const DF w = df_add(exact_diff(a1, a0), exact_diff(b0, b1));
+    if (fits_products(w.hi * w.hi)) {
+        s.add_product(w.hi, w.hi);
+        s.lo = fmaf(2.f * w.hi, w.lo, s.lo);
+    } else if (w.hi != 0.f) {
+        const double v = ((double)a1 - (double)a0) - ((double)b1 - (double)b0);
+        total += v * v;
+    }
+}
+__device__ __forceinline__ void add_square_of_curl(Sum<double> &s, double &, double a1, double a0, double b1, double b0)
+{
+    const double w = (a1 - a0) - (b1 - b0);
+    s.add_product(w, w);
+}
+
+template <typename T, int L, bool WALLS>
+__global__ void __launch_bounds__(ENS_THREADS, ENS_PER_SM)
+    k_enstrophy(Planes<T> P, double *partial, Geo g, Coll<typename Storage<T>::R> p, int planes)
+{
+    using R = typename Storage<T>::R;
+    __shared__ R su[2][3][ENS_THREADS];
     __shared__ double sh[32];
+    const int tid = threadIdx.x, lane = tid % ENS_LANES, row = tid / ENS_LANES;
+    const int ntx = (g.nx + ENS_X - 1) / ENS_X, nty = (g.ny + ENS_Y - 1) / ENS_Y, ntz = (g.nz + planes - 1) / planes;
+    const long long tiles = (long long)ntx * nty * ntz;
     double acc = 0.0;
-    const long long nxy = (long long)g.nx * g.ny;
-    const int n[3] = {g.nx, g.ny, g.nz};
-    const bool wall[3] = {g.wall_x != 0, g.wall_y != 0, g.wall_z != 0};
-    for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncell;
-         cell += (long long)gridDim.x * blockDim.x) {
-        const int z = (int)(cell / nxy);
-        const int rem = (int)(cell - z * nxy);
-        const int y = rem / g.nx;
-        const int x = rem - y * g.nx;
-        const int pos[3] = {x, y, z};
-        double own[3];
-        velocity_at<T, L>(grid, x, y, z, g, p, own);
-        // D[a][i] = (u_i(x + e_a) - u_i(x - e_a)) / 2
-        double D[3][3];
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int tx = (int)(t % ntx), ty = (int)(t / ntx % nty), tz = (int)(t / ntx / nty);
+        const int xr = tx * ENS_X - 1 + lane, yr = ty * ENS_Y - 1 + row;
+        const int z0 = tz * planes, z1 = min(z0 + planes, g.nz);
+        // this thread's column, wrapped; beyond the halo it repeats some column of the lattice
+        const int x = (xr + g.nx) % g.nx, y = (yr + g.ny) % g.ny;
+        const bool own = lane >= 1 && lane <= ENS_X && row >= 1 && row <= ENS_Y && xr < g.nx && yr < g.ny;
+        auto velocity = [&](int z, R u[3]) {
+            R f[Q];
+            gather_state<L>(P, Site<WALLS>(x, y, z < 0 ? z + g.nz : (z >= g.nz ? z - g.nz : z), 1, g), f);
+            R drho, rho0;
+            macro(f, p, drho, rho0, u);
+        };
+        R um[3], uc[3], up[3];
+        velocity(z0 - 1, um);
+        velocity(z0, uc);
+        Sum<R> s;
+        for (int z = z0; z < z1; ++z) {
+            const int b = z & 1;  // the other buffer may still be read for the plane before
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double up[3], um[3];
-            int qp[3] = {x, y, z}, qm[3] = {x, y, z};
-            const bool wp = wall[a] && pos[a] == n[a] - 1, wm = wall[a] && pos[a] == 0;
-            qp[a] = pos[a] == n[a] - 1 ? 0 : pos[a] + 1;
-            qm[a] = pos[a] == 0 ? n[a] - 1 : pos[a] - 1;
-            if (wp) { up[0] = -own[0]; up[1] = -own[1]; up[2] = -own[2]; }
-            else velocity_at<T, L>(grid, qp[0], qp[1], qp[2], g, p, up);
-            if (wm) { um[0] = -own[0]; um[1] = -own[1]; um[2] = -own[2]; }
-            else velocity_at<T, L>(grid, qm[0], qm[1], qm[2], g, p, um);
+            for (int i = 0; i < 3; ++i) su[b][i][tid] = uc[i];
+            velocity(z + 1, up);
+            __syncthreads();
+            if (own) {
+                // neighbours' velocities; a walled axis' ghost is -u of the own cell
+                auto nb = [&](int i, int at, bool wall) { return wall ? -uc[i] : su[b][i][at]; };
+                const bool wxm = g.wall_x && x == 0, wxp = g.wall_x && x == g.nx - 1;
+                const bool wym = g.wall_y && y == 0, wyp = g.wall_y && y == g.ny - 1;
+                const bool wzm = g.wall_z && z == 0, wzp = g.wall_z && z == g.nz - 1;
+                const R zm0 = wzm ? -uc[0] : um[0], zm1 = wzm ? -uc[1] : um[1];
+                const R zp0 = wzp ? -uc[0] : up[0], zp1 = wzp ? -uc[1] : up[1];
+                // 2 (d_y u_z - d_z u_y), 2 (d_z u_x - d_x u_z), 2 (d_x u_y - d_y u_x)
+                add_square_of_curl(s, acc, nb(2, tid + ENS_LANES, wyp), nb(2, tid - ENS_LANES, wym), zp1, zm1);
+                add_square_of_curl(s, acc, zp0, zm0, nb(2, tid + 1, wxp), nb(2, tid - 1, wxm));
+                add_square_of_curl(s, acc, nb(1, tid + 1, wxp), nb(1, tid - 1, wxm), nb(0, tid + ENS_LANES, wyp),
+                                   nb(0, tid - ENS_LANES, wym));
+            }
+            if ((z - z0) % SUM_CELLS == SUM_CELLS - 1) s.flush(acc);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) D[a][i] = 0.5 * (up[i] - um[i]);
+            for (int i = 0; i < 3; ++i) {
+                um[i] = uc[i];
+                uc[i] = up[i];
+            }
         }
-        const double wx = D[1][2] - D[2][1];
-        const double wy = D[2][0] - D[0][2];
-        const double wz = D[0][1] - D[1][0];
-        acc += wx * wx + wy * wy + wz * wz;
+        s.flush(acc);
+        __syncthreads();
     }
     const double v = block_sum(acc, sh);
-    if (threadIdx.x == 0) partial[blockIdx.x * 8] = v;
+    if (tid == 0) partial[blockIdx.x * 8] = v;
 }
 
 __global__ void __launch_bounds__(RED_THREADS) k_enstrophy_final(const double *partial, int nblocks,
@@ -244,7 +431,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_enstrophy_final(const double *p
     double v = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partial[b * 8];
     v = block_sum(v, sh);
-    if (threadIdx.x == 0) result[0] = 0.5 * v / ncell;
+    if (threadIdx.x == 0) result[0] = 0.125 * v / ncell;  // (twice the curl)^2, and 1/2
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -276,21 +463,17 @@ cudaError_t launch_moments(int prec, int layout, const void *grid, void *rho, vo
 {
     return by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        using R = typename Storage<T>::R;
-        Coll<R> p = to_coll<R>(cb);
-        const T *gr = (const T *)grid;
-        if (dtype == 0) {
-            double *r = (double *)rho, *uu = (double *)u;
-            if (layout == AB) k_moments<T, double, AB><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-            else if (layout == AA_EVEN) k_moments<T, double, AA_EVEN><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-            else k_moments<T, double, AA_ODD><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-        } else {
-            float *r = (float *)rho, *uu = (float *)u;
-            if (layout == AB) k_moments<T, float, AB><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-            else if (layout == AA_EVEN) k_moments<T, float, AA_EVEN><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-            else k_moments<T, float, AA_ODD><<<cell_blocks(g), CELL_THREADS, 0, s>>>(gr, r, uu, g, p, cell_box(g));
-        }
-        return cudaGetLastError();
+        const auto p = to_coll<typename Storage<T>::R>(cb);
+        const Planes<T> P = planes_of<T>(const_cast<void *>(grid), g.ncell);
+        const Box box = cell_box(g);
+        return by_layout(layout, g, [&](auto l, auto w) {
+            constexpr int L = decltype(l)::value;
+            constexpr bool W = decltype(w)::value;
+            if (dtype == 0)
+                k_moments<T, double, L, W><<<cell_blocks(g), CELL_THREADS, 0, s>>>(P, (double *)rho, (double *)u, g, p, box);
+            else
+                k_moments<T, float, L, W><<<cell_blocks(g), CELL_THREADS, 0, s>>>(P, (float *)rho, (float *)u, g, p, box);
+        });
     });
 }
 
@@ -324,13 +507,12 @@ cudaError_t launch_reduce(int prec, int layout, const void *grid, double *scratc
 {
     cudaError_t e = by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        using R = typename Storage<T>::R;
-        Coll<R> p = to_coll<R>(cb);
-        const T *gr = (const T *)grid;
-        if (layout == AB) k_reduce<T, AB><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        else if (layout == AA_EVEN) k_reduce<T, AA_EVEN><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        else k_reduce<T, AA_ODD><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        return cudaGetLastError();
+        const auto p = to_coll<typename Storage<T>::R>(cb);
+        const Planes<T> P = planes_of<T>(const_cast<void *>(grid), g.ncell);
+        const Box box = cell_box(g);
+        return by_layout(layout, g, [&](auto l, auto w) {
+            k_reduce<T, decltype(l)::value, decltype(w)::value><<<RED_BLOCKS, RED_THREADS, 0, s>>>(P, scratch, g, p, box);
+        });
     });
     if (e != cudaSuccess) return e;
     k_reduce_final<<<1, RED_THREADS, 0, s>>>(scratch, RED_BLOCKS, result, (double)g.ncell);
@@ -364,18 +546,18 @@ int reduce_noalloc_capacity_doubles() { return NOALLOC_DOUBLES; }
 cudaError_t launch_enstrophy(int prec, int layout, const void *grid, double *scratch, double *result, const Geo &g,
                              const CollBoth &c, cudaStream_t s)
 {
+    constexpr int blocks = RED_SMS * ENS_PER_SM;
     cudaError_t e = by_prec(prec, [&](auto tag) {
         using T = decltype(tag);
-        using R = typename Storage<T>::R;
-        const Coll<R> p = to_coll<R>(c);
-        const T *gr = static_cast<const T *>(grid);
-        if (layout == AB) k_enstrophy<T, AB><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        else if (layout == AA_EVEN) k_enstrophy<T, AA_EVEN><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        else k_enstrophy<T, AA_ODD><<<RED_BLOCKS, RED_THREADS, 0, s>>>(gr, scratch, g, p);
-        return cudaGetLastError();
+        const auto p = to_coll<typename Storage<T>::R>(c);
+        const Planes<T> P = planes_of<T>(const_cast<void *>(grid), g.ncell);
+        const int planes = enstrophy_planes(g);
+        return by_layout(layout, g, [&](auto l, auto w) {
+            k_enstrophy<T, decltype(l)::value, decltype(w)::value><<<blocks, ENS_THREADS, 0, s>>>(P, scratch, g, p, planes);
+        });
     });
     if (e != cudaSuccess) return e;
-    k_enstrophy_final<<<1, RED_THREADS, 0, s>>>(scratch, RED_BLOCKS, result, (double)g.ncell);
+    k_enstrophy_final<<<1, RED_THREADS, 0, s>>>(scratch, blocks, result, (double)g.ncell);
     return cudaGetLastError();
 }
 
