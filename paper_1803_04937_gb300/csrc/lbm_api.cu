@@ -87,8 +87,12 @@ lbm::Geo geo(const lbm_ctx *h)
 // lattice over more SMs and leave shorter tails (FP32 A/B, 256 -> 128 threads:
 // 16^3 2.18 -> 1.80 us, 80^3 9.78 -> 9.49; AA 96^3 15.2 -> 14.4; 256^3 unchanged),
 // and FP64, bound by its arithmetic, balances best by single warps (16^3 12.2 -> 6.2 us,
-// 32^3 12.3 -> 11.0).
-int block_threads(const lbm_ctx *h) { return h->precision == LBM_F64 ? 32 : 128; }
+// 32^3 12.3 -> 11.0).  Large D3Q27 lattices keep 256 (256^3 FP32 541 -> 537 us).
+int block_threads(const lbm_ctx *h)
+{
+    if (h->precision == LBM_F64) return 32;
+    return h->stencil == LBM_D3Q27 && ncell(h) >= (1 << 20) ? 256 : 128;
+}
 
 double omega_minus(const lbm_ctx *h)
 {

@@ -174,17 +174,24 @@ __device__ __forceinline__ void collide27(R g[Q27], const Relax27<R> &p)
     }
 }
 
-// A/B pull step, one cell per thread.
-template <typename T, bool RHO0, bool WALLS>
-__global__ void __launch_bounds__(256) k27_ab1(const T *__restrict__ src, T *__restrict__ dst, Geo g,
+// A/B pull step, one cell per thread.  FLAT: the cells as one sequence, or in
+// blocks that are rectangles of rows, which is faster with walls where rows fill
+// them (256^3 FP32: 538 -> 524 us) and slower without.
+template <typename T, bool RHO0, bool WALLS, bool FLAT = true>
+__global__ void __launch_bounds__(256) k27_ab1(const T *src, T *dst, Geo g,
                                                Relax27<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= box.count) return;
     int x, y, z;
-    box.at(i, x, y, z);
+    if constexpr (FLAT) {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= box.count) return;
+        box.at(i, x, y, z);
+    } else if (!box.at_block(x, y, z)) {
+        return;
+    }
     const Site<WALLS> s(x, y, z, 1, g);
+    step_begin(box);
     R f[Q27];
 #pragma unroll
     for (int q = 0; q < Q27; ++q) {
@@ -211,15 +218,21 @@ __global__ void __launch_bounds__(256) k27_ab1(const T *__restrict__ src, T *__r
 // A/B pull step for 16-bit storage, four cells per thread (nx % 4 == 0): the
 // same windowed quads as the D3Q19 four-cell step (each +-x shifted window
 // formed by funnel shifts from the aligned quad and its aligned neighbour),
-// 27 populations.  Bitwise the same results as k27_ab1.
-template <typename T, bool RHO0, bool WALLS, bool XONLY = false>
-__global__ void __launch_bounds__(128, 4) k27_ab4(const T *__restrict__ src, T *__restrict__ dst, Geo g,
+// 27 populations.  Bitwise the same results as k27_ab1.  FLAT as in k_aa_odd4
+// (256^3 FP16: 280 -> 268 us in rectangles).
+template <typename T, bool RHO0, bool WALLS, bool XONLY = false, bool FLAT = true>
+__global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g,
                                                   Relax27<float> p, Box box)
 {
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= box.count) return;
     int xq, y, z;
-    box.at(i, xq, y, z);
+    if constexpr (FLAT) {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= box.count) return;
+        if constexpr (WALLS && !XONLY) box.at_wall(i, xq, y, z);
+        else box.at(i, xq, y, z);
+    } else if (!box.at_block(xq, y, z)) {
+        return;
+    }
     const int x0 = 4 * xq;
     Site<WALLS> s(x0, y, z, 4, g);
     drop_yz<XONLY>(s);
@@ -243,7 +256,7 @@ __global__ void __launch_bounds__(128, 4) k27_ab4(const T *__restrict__ src, T *
         const uint2 *pn = reinterpret_cast<const uint2 *>(plane + (cx > 0 ? xprev : xnext));
         const bool xwall = WALLS && ((cx > 0 && s.bxm) || (cx < 0 && s.bxp));
         if (xwall && !w) pn = reinterpret_cast<const uint2 *>(bnc + x0);
-        win[q] = __ldg(pq);
+        win[q] = __ldg(pq);  // so not launched early (launch_step_kernel)
         if (cx != 0) nb[q] = w ? make_uint2(0u, 0u) : __ldg(pn);
     }
 #pragma unroll
@@ -282,6 +295,7 @@ __global__ void __launch_bounds__(128, 4) k27_ab4(const T *__restrict__ src, T *
 #pragma unroll
     for (int q = 0; q < Q27; ++q)
         *reinterpret_cast<uint2 *>(out + (long long)q * g.ncell + s.own + x0) = win[q];
+    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // Writes the canonical populations fc (f_q(x) - w_q) of cell x into an A/B
@@ -448,15 +462,13 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
                 // of the copy bandwidth
                 auto run = [&](auto rho0, auto walled) {
                     constexpr bool RH = decltype(rho0)::value, W = decltype(walled)::value;
-                    split_rows<W>(g, [&](int kind, int y0, int y1, int z0, int planes) {
-                        const Box box(g.nx / 4, y0, y1, z0, planes);
-                        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
-                        if (kind == ROWS_WALLED)
-                            q27::k27_ab4<T, RH, true><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
-                        else if (kind == ROWS_XWALLS)
-                            q27::k27_ab4<T, RH, true, true><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
-                        else
-                            q27::k27_ab4<T, RH, false><<<grid, QUAD_THREADS, 0, stream>>>(a, b, g, p, box);
+                    split_rows<W>(g, g.nx / 4, [&](int kind, const Box &box) {
+                        const int bx = kind == ROWS_WALLED ? 0 : box.block_x(QUAD_THREADS);
+                        auto k = kind == ROWS_WALLED ? q27::k27_ab4<T, RH, true>
+                                 : kind == ROWS_XWALLS
+                                     ? (bx ? q27::k27_ab4<T, RH, true, true, false> : q27::k27_ab4<T, RH, true, true>)
+                                     : (bx ? q27::k27_ab4<T, RH, false, false, false> : q27::k27_ab4<T, RH, false>);
+                        launch_step_box(k, box.beside, box, bx, QUAD_THREADS, stream, a, b, g, p);
                     });
                 };
                 if (c.rho0_is_rho && walls) run(std::true_type{}, std::true_type{});
@@ -466,16 +478,15 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
                 return cudaGetLastError();
             }
         }
-        const int bl = s.threads;
-        const unsigned gr = blocks_for(g.ncell, bl);
         const Box box = q27_box(g);
-        if (c.rho0_is_rho) {
-            if (walls) q27::k27_ab1<T, true, true><<<gr, bl, 0, stream>>>(a, b, g, p, box);
-            else q27::k27_ab1<T, true, false><<<gr, bl, 0, stream>>>(a, b, g, p, box);
-        } else {
-            if (walls) q27::k27_ab1<T, false, true><<<gr, bl, 0, stream>>>(a, b, g, p, box);
-            else q27::k27_ab1<T, false, false><<<gr, bl, 0, stream>>>(a, b, g, p, box);
-        }
+        const int bx = walls && s.threads >= 128 ? box.block_x(s.threads) : 0;
+        auto k = c.rho0_is_rho ? (bx      ? q27::k27_ab1<T, true, true, false>
+                                  : walls ? q27::k27_ab1<T, true, true>
+                                          : q27::k27_ab1<T, true, false>)
+                               : (bx      ? q27::k27_ab1<T, false, true, false>
+                                  : walls ? q27::k27_ab1<T, false, true>
+                                          : q27::k27_ab1<T, false, false>);
+        launch_step_box(k, true, box, bx, s.threads, stream, a, b, g, p);
         return cudaGetLastError();
     });
 }

@@ -70,6 +70,7 @@ template <> struct Storage<__nv_bfloat16> {
 
 // ---------------------------------------------------------------- geometry
 
+
 struct Geo {
     int nx, ny, nz;
     int wall_x, wall_y, wall_z;  // 1: half-way bounce-back walls at both ends
@@ -110,11 +111,16 @@ struct Box {
     unsigned count;  // items
     int y0, z0;
     Divider per_row, rows;  // items in a row, rows in a plane of the box
+    int y_walled = 0;       // wall rows only: rows of the faces normal to y, which come first
+    Divider planes{1};      // ... and planes of a y face
+    int y_last = 0, z_last = 0;
+    int nz = 0;             // planes of the box
+    bool beside = false;    // runs beside the launch before it (see step_begin)
 
     Box() = default;
-    Box(int items_per_row, int y0_, int y1, int z0_, int nz)
-        : count((unsigned)((long long)items_per_row * (y1 - y0_) * nz)), y0(y0_), z0(z0_), per_row(items_per_row),
-          rows(y1 - y0_)
+    Box(int items_per_row, int y0_, int y1, int z0_, int planes_)
+        : count((unsigned)((long long)items_per_row * (y1 - y0_) * planes_)), y0(y0_), z0(z0_),
+          per_row(items_per_row), rows(y1 - y0_), nz(planes_)
     {
     }
     // item i: its place in the row, y and z
@@ -124,7 +130,84 @@ struct Box {
         z = z0 + rows.div(per_row.div((int)i, item), yr);
         y = y0 + yr;
     }
+
+    // the same from a thread's place in a grid of blocks that are rectangles of
+    // rows; false for a thread outside the box
+    __device__ __forceinline__ bool at_block(int &item, int &y, int &z) const
+    {
+        item = blockIdx.x * blockDim.x + threadIdx.x;
+        const unsigned yr = blockIdx.y * blockDim.y + threadIdx.y;
+        y = y0 + (int)yr;
+        z = z0 + (int)blockIdx.z;
+        return item < (int)per_row.d && yr < rows.d;
+    }
+    // Threads along x of such blocks, 128, 64 or 32 of `threads`, with the fewest
+    // idle lanes at the end of a row, the larger on ties; 0: take the items as one
+    // sequence, because more than 1/8 of the lanes would be idle or the grid would
+    // have too many rows.
+    int block_x(int threads) const
+    {
+        const int n = (int)per_row.d;
+        int bx = 0, idle = 0;
+        for (int c = 128; c >= 32; c /= 2) {
+            const int w = (n + c - 1) / c * c - n;
+            if (c <= threads && (!bx || w < idle)) {
+                bx = c;
+                idle = w;
+            }
+        }
+        const long long by = threads / bx;
+        return 8LL * idle > n || (rows.d + by - 1) / by > 65535 ? 0 : bx;
+    }
+
+    // The rows at walls normal to y or z: rows y = 0 and ny - 1 over all z, then
+    // planes z = 0 and nz - 1 over the other y.
+    static Box wall_rows(int items_per_row, const Geo &g)
+    {
+        const int ylo = g.wall_y ? 1 : 0, yhi = g.wall_y ? g.ny - 1 : g.ny;
+        Box b;
+        b.y0 = ylo;
+        b.z0 = 0;
+        b.per_row = Divider(items_per_row);
+        b.rows = Divider(yhi > ylo ? yhi - ylo : 1);
+        b.planes = Divider(g.nz);
+        b.y_last = g.ny - 1;
+        b.z_last = g.nz - 1;
+        b.y_walled = g.wall_y ? (g.ny > 1 ? 2 : 1) * g.nz : 0;
+        const long long z_walled = g.wall_z && yhi > ylo ? (long long)(g.nz > 1 ? 2 : 1) * (yhi - ylo) : 0;
+        b.count = (unsigned)(items_per_row * (b.y_walled + z_walled));
+        return b;
+    }
+    __device__ __forceinline__ void at_wall(unsigned i, int &item, int &y, int &z) const
+    {
+        const int row = per_row.div((int)i, item);
+        if (row < y_walled) {
+            y = planes.div(row, z) ? y_last : 0;
+        } else {
+            int yr;
+            z = rows.div(row - y_walled, yr) ? z_last : 0;
+            y = y0 + yr;
+        }
+    }
 };
+
+// Launches of consecutive steps overlap their start with the end of the one
+// before (programmatic dependent launch): a step's blocks may be scheduled once
+// all blocks of the launch before have passed step_begin, that is once it needs
+// no more slots, and wait there for its completion.  A launch `beside` the one
+// before works on other rows of the same step: it reads what the step before
+// left, which the launch beside it has waited for, so it need not wait for that
+// one before its work but only before it ends, so that its own completion stands
+// for both.
+__device__ __forceinline__ void step_begin(const Box &box)
+{
+    if (!box.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void step_end(const Box &box)
+{
+    if (box.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // One lattice cell with its wrapped neighbour coordinates and the wall flags
 // of its six faces (true when the neighbour across that face is beyond a wall).

@@ -29,6 +29,7 @@
 #pragma once
 
 #include <type_traits>
+#include <utility>
 
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(256) k_ab1(Planes<T> src, Planes<T> dst, Geo g
     if (i >= box.count) return;
     int x, y, z;
     box.at(i, x, y, z);
+    step_begin(box);
     if constexpr (WALLS) {
         // warps with no cell at a wall take the periodic body (uniform branch per warp)
         const Site<true> sw(x, y, z, 1, g);
@@ -261,11 +263,12 @@ constexpr int aa1_blocks(bool odd)
 // the stores (80 instead of 40 registers; +1.5 % FP32, +2.8 % FP64 measured).
 template <typename T, bool RHO0, bool MRT = false>
 __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(false)) k_aa_even1(Planes<T> P, Planes<T> Pw, Geo g,
-                                                                           Relax<typename Storage<T>::R> p)
+                                                                           Relax<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
     const unsigned own = blockIdx.x * blockDim.x + threadIdx.x;
     if (own >= (unsigned)g.ncell) return;
+    step_begin(box);
     R f[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) f[q] = Storage<T>::load(P.p[q] + own);
@@ -285,7 +288,9 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Plane
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= box.count) return;
     int x, y, z;
-    box.at(i, x, y, z);
+    if constexpr (WALLS && !XONLY) box.at_wall(i, x, y, z);
+    else box.at(i, x, y, z);
+    step_begin(box);
     Site<WALLS> s(x, y, z, 1, g);
     drop_yz<XONLY>(s);
     R f[Q];
@@ -303,6 +308,7 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Plane
         T *a = w ? P.p[OPP(q)] + s.own + x : P.p[q] + s.template row_along<1>(q) + xt;
         Storage<T>::store(a, f[q]);
     }
+    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // ---------------------------------------------------------------- two cells per thread
@@ -529,12 +535,14 @@ __device__ __forceinline__ void load4w(const Planes<T> &P, const Site<WALLS> &s,
         const uint2 *pn = reinterpret_cast<const uint2 *>(srcq + srow + (cx > 0 ? xprev : xnext));
         const bool xwall = WALLS && ((cx > 0 && s.bxm) || (cx < 0 && s.bxp));
         if (xwall && !w) pn = reinterpret_cast<const uint2 *>(bncq + s.own + xs);
-        // Non-coherent loads, also in the in-place AA odd step (SWAP): the
-        // elements it uses of a quad are its own cells' inputs, which only this
-        // thread writes, and only after it has read them; the other elements of
-        // a neighbour quad may be stale there and are not used.
-        win[q] = __ldg(pq);
-        if (cx != 0) nb[q] = w ? make_uint2(0u, 0u) : __ldg(pn);
+        // The in-place AA odd step (SWAP) takes non-coherent loads (FP16 0.797 -> 0.803,
+        // BF16 0.774 -> 0.791 of the copy bandwidth at 256^3): the elements it uses of
+        // a quad are its own cells' inputs, which only this thread writes, and only
+        // after it has read them; the other elements of a neighbour quad may be stale
+        // and are not used.  Such a launch must not start before the end of the one
+        // whose results it reads (launch_step_kernel).
+        win[q] = SWAP ? __ldg(pq) : *pq;
+        if (cx != 0) nb[q] = w ? make_uint2(0u, 0u) : (SWAP ? __ldg(pn) : *pn);
     }
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
@@ -614,26 +622,13 @@ __global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Pla
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= box.count) return;  // no lane needs another lane's data
     int xq, y, z;
-    box.at(i, xq, y, z);
-    const int x0 = 4 * xq;
-    if constexpr (XONLY) {
-        Site<true> sx(x0, y, z, 4, g);
-        drop_yz<true>(sx);
-        ab4_body<T, RHO0, true, MRT>(src, dst, sx, g, p);
-        return;
-    }
-    if constexpr (WALLS) {
-        // A warp covers one row segment; where none of its cells touches a wall
-        // (all but the wall rows and the row ends) it takes the periodic body,
-        // which has no bounce-back selects.  The branch is uniform per warp.
-        const Site<true> sw(x0, y, z, 4, g);
-        const bool touches = sw.bxm || sw.bxp || sw.bym || sw.byp || sw.bzm || sw.bzp;
-        if (__any_sync(__activemask(), touches)) {
-            ab4_body<T, RHO0, true, MRT>(src, dst, sw, g, p);
-            return;
-        }
-    }
-    ab4_body<T, RHO0, false, MRT>(src, dst, Site<false>(x0, y, z, 4, g), g, p);
+    if constexpr (WALLS && !XONLY) box.at_wall(i, xq, y, z);
+    else box.at(i, xq, y, z);
+    Site<WALLS> s(4 * xq, y, z, 4, g);
+    drop_yz<XONLY>(s);
+    step_begin(box);
+    ab4_body<T, RHO0, WALLS, MRT>(src, dst, s, g, p);
+    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // AA even step for 16-bit storage, four cells per thread: own quads of plane
@@ -641,11 +636,12 @@ __global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Pla
 // plane table (see k_aa_even1), which lets the step run five blocks per SM
 // without spills (96 registers; with one table it needed 128).
 template <typename T, bool RHO0, bool MRT = false>
-__global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, Geo g, Relax<float> p)
+__global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, Geo g, Relax<float> p, Box box)
 {
-    const long long first = 4LL * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
-    if (first >= g.ncell) return;
-    const int own = (int)first;
+    int own = 4 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if ((unsigned)own >= (unsigned)g.ncell) return;
+    opaque(own);  // (left to see through it, the compiler spills 96 bytes)
+    step_begin(box);
     uint2 quad[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q)
@@ -669,19 +665,43 @@ __global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, 
 // quad goes to plane qbar of the own cells.  Each location is written by one
 // thread, and read (for a value that is used) only by that thread, as in the
 // one-cell kernel.
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
+// FORM: how the quads are walked.  ROWS_OF_BLOCKS: in blocks that are rectangles
+// of rows, whose rows a warp does not leave; the fastest from DRAM where rows fill
+// them (step of a pair, 256^3: FP16 208 us against 227, BF16 212 against 229).
+// SEQUENCE: as one sequence (192^3 FP16: 95 against 108 us, 160^3 60 against 74).
+// SEQUENCE_CACHED: the same for lattices that stay in L2 (128^3 FP16 22.8 against
+// 26.8 us); it differs in the branch before the loads, without which the compiler
+// spreads them among the collisions: that saves its spills, but leaves too few
+// loads in flight for DRAM (192^3 FP16: 99 us).
+enum OddForm { ROWS_OF_BLOCKS, SEQUENCE, SEQUENCE_CACHED };
+template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false, OddForm FORM = SEQUENCE>
 __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g, Relax<float> p, Box box)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool active = i < box.count;
+    constexpr bool SEQ = FORM != ROWS_OF_BLOCKS;
     int xq, y, z;
-    box.at(active ? i : box.count - 1u, xq, y, z);
+    bool active, end;  // end: the last quad there is for a warp that is not full
+    if constexpr (SEQ) {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        active = i < box.count;
+        end = i + 1 >= box.count;
+        if constexpr (WALLS && !XONLY) box.at_wall(active ? i : box.count - 1u, xq, y, z);
+        else box.at(active ? i : box.count - 1u, xq, y, z);
+    } else {
+        const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+        y = (WALLS ? box.y0 : 0) + (int)(blockIdx.y * blockDim.y + threadIdx.y);
+        z = (WALLS ? box.z0 : 0) + (int)blockIdx.z;
+        if (y >= (WALLS ? box.y0 + (int)box.rows.d : g.ny)) return;  // uniform across the warp
+        active = x0 < g.nx;
+        xq = active ? x0 >> 2 : 0;
+        end = false;
+    }
     Site<WALLS> s(4 * xq, y, z, 4, g);
     drop_yz<XONLY>(s);
-    // ends of the lanes' segment of a row (a warp may hold several rows' ends)
-    const bool head = lane == 0 || xq == 0;
-    const bool last = lane == 31 || s.x + 4 >= g.nx || i + 1 >= box.count;
+    // ends of the lanes' segment of a row (a warp of a sequence may hold several rows' ends)
+    const bool head = lane == 0 || (SEQ && xq == 0);
+    const bool last = lane == 31 || s.x + 4 >= g.nx || end;
+    if constexpr (FORM == SEQUENCE) step_begin(box);  // a branch that the loads stay behind; nothing to wait for
     uint2 quad[Q];
     load4w<true>(P, s, g, quad);
     if (active) collide4<T, RHO0, MRT>(quad, p);
@@ -738,48 +758,79 @@ __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g
                 *((WALLS && s.bxm) ? bnc + sw.own + sw.x : dst + trow + sw.xm) = (unsigned short)(quad[q].x & 0xffffu);
         }
     }
+    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // ---------------------------------------------------------------- dispatch
 
-// Calls launch(kind, rows, nz_rows) for the launches of one step.  A periodic
-// lattice is one ROWS_PERIODIC launch over all rows.  With walls, the interior
-// rows (no link crosses a y or z wall) run the periodic kernel, or with walls
-// on x the kernel that has the x-wall selects only (ROWS_XWALLS), and the wall
-// rows the walled one (ROWS_WALLED): rows y = 0 and ny - 1 over all z, then
-// planes z = 0 and nz - 1 over the interior y; every row is in exactly one
-// launch.  All kernels compute a cell with the same code as the single walled
-// launch, so the results are bitwise the same.  The walled four-cell kernel
-// carries both bodies and spills; keeping it to the wall rows took the walled
-// channel 512x256x256 from 84.3 to 89.1 GLUPS (FP16) and from 80.0 to 86.9
-// (BF16), and a cavity (walls on x, y and z) 512x256x256 from 0.76 to 0.95 of
-// the copy bandwidth (FP16 A/B).
 // Kinds of the launches of split_rows.
 enum { ROWS_PERIODIC = 0, ROWS_WALLED = 1, ROWS_XWALLS = 2 };
 
-// launch(kind, y0, y1, z0, planes)
+// Calls launch(kind, box) for the launches of one step.  A periodic lattice is
+// one ROWS_PERIODIC launch over all rows.  With walls, the interior rows (no
+// link crosses a y or z wall) run the periodic kernel, or with walls on x the
+// kernel that has the x-wall selects only (ROWS_XWALLS), and the rows at y and z
+// walls the walled one (ROWS_WALLED) in one launch beside it; every row is in
+// exactly one launch, and no launch reads what the other writes.  All kernels
+// compute a cell with the same code, so the results are bitwise the same.  A
+// walled four-cell kernel over all rows carries both bodies and spills; keeping
+// it to the wall rows took the walled channel 512x256x256 from 84.3 to 89.1
+// GLUPS (FP16) and from 80.0 to 86.9 (BF16), and a cavity (walls on x, y and z)
+// 512x256x256 from 0.76 to 0.95 of the copy bandwidth (FP16 A/B).  One launch
+// for all wall rows that runs beside the interior one, instead of four after it:
+// closed box 32^3 FP16 A/B 14.2 -> 3.7 us a step, 128^3 41.3 -> 28.3.
 template <bool WALLS, typename F>
-static void split_rows(const Geo &g, F &&launch)
+static void split_rows(const Geo &g, int items_per_row, F &&launch)
 {
     if (!WALLS) {
-        launch(ROWS_PERIODIC, 0, g.ny, 0, g.nz);
+        launch(ROWS_PERIODIC, Box(items_per_row, 0, g.ny, 0, g.nz));
         return;
     }
-    const int inner = g.wall_x ? ROWS_XWALLS : ROWS_PERIODIC;
     const int ylo = g.wall_y ? 1 : 0, yhi = g.wall_y ? g.ny - 1 : g.ny;
     const int zlo = g.wall_z ? 1 : 0, zhi = g.wall_z ? g.nz - 1 : g.nz;
-    if (yhi > ylo && zhi > zlo) launch(inner, ylo, yhi, zlo, zhi - zlo);
-    if (g.wall_y) {
-        launch(ROWS_WALLED, 0, 1, 0, g.nz);
-        if (g.ny > 1) launch(ROWS_WALLED, g.ny - 1, g.ny, 0, g.nz);
-    }
-    if (g.wall_z && yhi > ylo) {
-        launch(ROWS_WALLED, ylo, yhi, 0, 1);
-        if (g.nz > 1) launch(ROWS_WALLED, ylo, yhi, g.nz - 1, 1);
-    }
+    const bool interior = yhi > ylo && zhi > zlo;
+    if (interior) launch(g.wall_x ? ROWS_XWALLS : ROWS_PERIODIC, Box(items_per_row, ylo, yhi, zlo, zhi - zlo));
+    Box walls = Box::wall_rows(items_per_row, g);
+    walls.beside = interior;
+    if (walls.count) launch(ROWS_WALLED, walls);
 }
 
 static inline unsigned blocks_for(long long items, int threads) { return (unsigned)((items + threads - 1) / threads); }
+
+// Launches a step kernel; early: as a programmatic dependent of the stream's
+// last launch (step_begin).  Kernels with non-coherent loads are not launched
+// early, except beside a launch of the same step that was not, whose start
+// already followed the end of the step before.
+template <typename... P, typename... A>
+static void launch_step_kernel(void (*kernel)(P...), bool early, dim3 grid, dim3 threads, cudaStream_t stream,
+                               A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = threads;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);  // its error is the caller's cudaGetLastError
+}
+
+// ... over a box, whose rows fill blocks of bx threads along x, or (bx = 0) as
+// one sequence of items; the box is the kernel's last argument.
+template <typename... P, typename... A>
+static void launch_step_box(void (*kernel)(P...), bool early, const Box &box, int bx, int threads, cudaStream_t stream,
+                            A &&...args)
+{
+    if (bx == 0) {
+        launch_step_kernel(kernel, early, blocks_for(box.count, threads), threads, stream, std::forward<A>(args)..., box);
+        return;
+    }
+    const unsigned ux = (unsigned)bx, uy = (unsigned)(threads / bx);
+    launch_step_kernel(kernel, early, dim3((box.per_row.d + ux - 1) / ux, (box.rows.d + uy - 1) / uy, (unsigned)box.nz),
+                       dim3(ux, uy), stream, std::forward<A>(args)..., box);
+}
 
 // The one-cell A/B step stays one launch over all rows: its walled kernel
 // already runs at the periodic kernel's speed (walled channel 512x256x256,
@@ -789,7 +840,7 @@ static void launch_ab1(const Planes<T> &S, const Planes<T> &D, const Geo &g, con
                        int threads, cudaStream_t stream)
 {
     const Box box(g.nx, 0, g.ny, 0, g.nz);
-    k_ab1<T, RHO0, WALLS, MRT><<<blocks_for(box.count, threads), threads, 0, stream>>>(S, D, g, p, box);
+    launch_step_box(k_ab1<T, RHO0, WALLS, MRT>, true, box, 0, threads, stream, S, D, g, p);
 }
 
 // The one-cell AA odd step, split into interior and wall rows like the
@@ -799,15 +850,11 @@ template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_aa_odd1(const Planes<T> &P, const Geo &g, const Relax<typename Storage<T>::R> &p, int threads,
                            cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
-        const Box box(g.nx, y0, y1, z0, planes);
-        const unsigned grid = blocks_for(box.count, threads);
-        if (kind == ROWS_WALLED)
-            k_aa_odd1<T, RHO0, true, MRT><<<grid, threads, 0, stream>>>(P, g, p, box);
-        else if (kind == ROWS_XWALLS)
-            k_aa_odd1<T, RHO0, true, MRT, true><<<grid, threads, 0, stream>>>(P, g, p, box);
-        else
-            k_aa_odd1<T, RHO0, false, MRT><<<grid, threads, 0, stream>>>(P, g, p, box);
+    split_rows<WALLS>(g, g.nx, [&](int kind, const Box &box) {
+        auto k = kind == ROWS_WALLED   ? k_aa_odd1<T, RHO0, true, MRT>
+                 : kind == ROWS_XWALLS ? k_aa_odd1<T, RHO0, true, MRT, true>
+                                       : k_aa_odd1<T, RHO0, false, MRT>;
+        launch_step_box(k, true, box, 0, threads, stream, P, g, p);
     });
 }
 
@@ -816,15 +863,11 @@ constexpr int QUAD_THREADS = 128;  // threads per block of the four-cell kernels
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
-        const Box box(g.nx / 4, y0, y1, z0, planes);
-        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
-        if (kind == ROWS_WALLED)
-            k_ab4<T, RHO0, true, MRT><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
-        else if (kind == ROWS_XWALLS)
-            k_ab4<T, RHO0, true, MRT, true><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
-        else
-            k_ab4<T, RHO0, false, MRT><<<grid, QUAD_THREADS, 0, stream>>>(S, D, g, p, box);
+    split_rows<WALLS>(g, g.nx / 4, [&](int kind, const Box &box) {
+        auto k = kind == ROWS_WALLED   ? k_ab4<T, RHO0, true, MRT>
+                 : kind == ROWS_XWALLS ? k_ab4<T, RHO0, true, MRT, true>
+                                       : k_ab4<T, RHO0, false, MRT>;
+        launch_step_box(k, true, box, 0, QUAD_THREADS, stream, S, D, g, p);
     });
 }
 
@@ -836,19 +879,22 @@ static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, con
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_aa_odd4(const Planes<T> &P, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, [&](int kind, int y0, int y1, int z0, int planes) {
-        const Box box(g.nx / 4, y0, y1, z0, planes);
-        const unsigned grid = blocks_for(box.count, QUAD_THREADS);
+    split_rows<WALLS>(g, g.nx / 4, [&](int kind, const Box &box) {
+        // the form for grids that stay in L2 (129 MB, with the next step's share)
+        // serves periodic lattices only (128^3 with walls: 33.4 us, 29.1 in blocks)
+        const bool cached = !WALLS && g.ncell * Q * (long long)sizeof(T) < (100LL << 20);
+        const int bx = kind == ROWS_WALLED || cached ? 0 : box.block_x(QUAD_THREADS);
+        // BF16 takes that form for every sequence (192^3: 101 against 103 us)
+        constexpr OddForm seq = std::is_same_v<T, __nv_bfloat16> ? SEQUENCE_CACHED : SEQUENCE;
         // the interior rows of a walled lattice take the x-walls-only kernel also
         // without x walls (its x flags are then false): it compiles to a faster
         // step than the periodic kernel with a row range (walled channel, FP16 AA
         // pair 0.81 -> 0.85, BF16 0.80 -> 0.82)
-        if (kind == ROWS_WALLED)
-            k_aa_odd4<T, RHO0, true, MRT><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
-        else if (WALLS)
-            k_aa_odd4<T, RHO0, true, MRT, true><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
-        else
-            k_aa_odd4<T, RHO0, false, MRT><<<grid, QUAD_THREADS, 0, stream>>>(P, g, p, box);
+        auto k = kind == ROWS_WALLED ? k_aa_odd4<T, RHO0, true, MRT>
+                 : WALLS  ? (bx ? k_aa_odd4<T, RHO0, true, MRT, true, ROWS_OF_BLOCKS> : k_aa_odd4<T, RHO0, true, MRT, true>)
+                 : cached ? k_aa_odd4<T, RHO0, false, MRT, false, SEQUENCE_CACHED>
+                          : (bx ? k_aa_odd4<T, RHO0, false, MRT, false, ROWS_OF_BLOCKS> : k_aa_odd4<T, RHO0, false, MRT, false, seq>);
+        launch_step_box(k, box.beside, box, bx, QUAD_THREADS, stream, P, g, p);
     });
 }
 
@@ -860,7 +906,8 @@ static void launch_step1(int kind, void *src, const Planes<T> &D, const Geo &g,
     if (kind == 0)
         launch_ab1<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, threads, stream);
     else if (kind == 1)
-        k_aa_even1<T, RHO0, MRT><<<blocks_for(g.ncell, threads), threads, 0, stream>>>(D, D, g, p);
+        launch_step_kernel(k_aa_even1<T, RHO0, MRT>, true, blocks_for(g.ncell, threads), threads, stream, D, D, g, p,
+                           Box());
     else
         launch_aa_odd1<T, RHO0, WALLS, MRT>(D, g, p, threads, stream);
 }
@@ -873,7 +920,8 @@ static void launch_step4(int kind, void *src, const Planes<T> &D, const Geo &g, 
     if (kind == 0)
         launch_ab4<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, stream);
     else if (kind == 1)
-        k_aa_even4<T, RHO0, MRT><<<blocks_for(g.ncell / 4, QUAD_THREADS), QUAD_THREADS, 0, stream>>>(D, D, g, p);
+        launch_step_kernel(k_aa_even4<T, RHO0, MRT>, true, blocks_for(g.ncell / 4, QUAD_THREADS), QUAD_THREADS, stream, D,
+                           D, g, p, Box());
     else
         launch_aa_odd4<T, RHO0, WALLS, MRT>(D, g, p, stream);
 }
