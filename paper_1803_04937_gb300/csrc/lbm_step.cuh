@@ -313,16 +313,34 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Plane
 
 // ---------------------------------------------------------------- two cells per thread
 
+// The pair of a thread of a sequence of pairs (Box), and its place in the warp:
+// head / last pair of the warp's part of a row (a warp may hold several rows'
+// ends).  Threads past the end repeat the last pair and take part in the shuffles.
+struct PairAt {
+    int x0, y, z;
+    bool active, head, last;
+
+    __device__ __forceinline__ PairAt(const Box &box, bool wall_rows = false)
+    {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        const int lane = threadIdx.x & 31;
+        active = i < box.count;
+        int xp;
+        if (wall_rows) box.at_wall(active ? i : box.count - 1u, xp, y, z);
+        else box.at(active ? i : box.count - 1u, xp, y, z);
+        x0 = 2 * xp;
+        head = lane == 0 || xp == 0;
+        last = lane == 31 || xp + 1 == (int)box.per_row.d || i + 1 >= box.count;
+    }
+};
+
 // Pair-wise gather for the cells (x0, x0 + 1), x0 even, nx even (layouts as
-// in gather1).  blockDim.x is a multiple of 32, so a warp never spans two
-// lattice rows and lane 0 of a warp starts a 64-cell segment of its row.
-// Inactive lanes (x0 >= nx) read a valid pair and take part in the shuffles.
+// in gather1).
 template <bool SWAP, bool WALLS, typename T, typename R>
-__device__ __forceinline__ void gather2(const Planes<T> &P, const Site<WALLS> &s, const Geo &g, int lane,
-                                        bool active, R f0[Q], R f1[Q])
+__device__ __forceinline__ void gather2(const Planes<T> &P, const Site<WALLS> &s, const PairAt &at, R f0[Q], R f1[Q])
 {
     const int x0 = s.x;
-    const bool last = lane == 31 || x0 + 2 >= g.nx;
+    const bool active = at.active, last = at.last;
     // Phase 1: issue every load before any shuffle.  lo/hi: the own pair of
     // the source row (or, through a y/z wall, the own cell's reflected pair);
     // e: the element beyond the segment's edge for the +-x populations.
@@ -338,7 +356,7 @@ __device__ __forceinline__ void gather2(const Planes<T> &P, const Site<WALLS> &s
         e[q] = R(0);
         if (cx > 0) {  // pull from x - 1: lane 0 needs element x0 - 1
             const T *a = (WALLS && s.bxm) ? bnc + s.own + x0 : src + srow + s.xm;
-            if (lane == 0 && active && !w) e[q] = Storage<T>::load(a);
+            if (at.head && active && !w) e[q] = Storage<T>::load(a);
         } else if (cx < 0) {  // pull from x + 1: the segment's last lane needs element x0 + 2
             const T *a = (WALLS && s.bxp) ? bnc + s.own + x0 + 1 : src + srow + s.xp;
             if (last && active && !w) e[q] = Storage<T>::load(a);
@@ -354,7 +372,7 @@ __device__ __forceinline__ void gather2(const Planes<T> &P, const Site<WALLS> &s
             f1[q] = hi[q];
         } else if (cx > 0) {
             R left = __shfl_up_sync(0xffffffffu, hi[q], 1);
-            if (lane == 0) left = e[q];
+            if (at.head) left = e[q];
             f0[q] = w ? lo[q] : left;
             f1[q] = w ? hi[q] : lo[q];
         } else {
@@ -367,19 +385,17 @@ __device__ __forceinline__ void gather2(const Planes<T> &P, const Site<WALLS> &s
 }
 
 template <typename T, bool RHO0, bool WALLS>
-__global__ void __launch_bounds__(256, 4) k_ab2(Planes<T> src, Planes<T> dst, Geo g, Relax<typename Storage<T>::R> p)
+__global__ void __launch_bounds__(256, 4) k_ab2(Planes<T> src, Planes<T> dst, Geo g, Relax<typename Storage<T>::R> p,
+                                                Box box)
 {
     using R = typename Storage<T>::R;
-    const int lane = threadIdx.x & 31;
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (y >= g.ny) return;  // uniform across the warp
-    const bool active = x0 < g.nx;
-    const Site<WALLS> s(active ? x0 : 0, y, z, 2, g);
+    const PairAt at(box);
+    const Site<WALLS> s(at.x0, at.y, at.z, 2, g);
+    step_begin(box);
     R f0[Q], f1[Q];
-    gather2<false>(src, s, g, lane, active, f0, f1);
-    if (!active) return;
+    gather2<false>(src, s, at, f0, f1);
+    if (!at.active) return;
+    const int x0 = at.x0;
     collide_lean<R, RHO0, one_rounding_v<T>>(f0, p);
     collide_lean<R, RHO0, one_rounding_v<T>>(f1, p);
 #pragma unroll
@@ -387,14 +403,13 @@ __global__ void __launch_bounds__(256, 4) k_ab2(Planes<T> src, Planes<T> dst, Ge
 }
 
 template <typename T, bool RHO0>
-__global__ void __launch_bounds__(256) k_aa_even2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p)
+__global__ void __launch_bounds__(256) k_aa_even2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x0 >= g.nx || y >= g.ny) return;
-    const int own = (z * g.ny + y) * g.nx + x0;
+    int own = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if ((unsigned)own >= (unsigned)g.ncell) return;
+    opaque(own);
+    step_begin(box);
     R f0[Q], f1[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) Pair<T>::load(P.p[q] + own, f0[q], f1[q]);
@@ -411,24 +426,22 @@ __global__ void __launch_bounds__(256) k_aa_even2(Planes<T> P, Geo g, Relax<type
 // neighbouring segment is written by the edge lane as a scalar.  Through a
 // wall the value goes to plane qbar of the own cell.  Every location is
 // written by exactly one thread, as in the one-cell kernel.
-template <typename T, bool RHO0, bool WALLS>
-__global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p)
+template <typename T, bool RHO0, bool WALLS, bool XONLY = false>
+__global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
-    const int lane = threadIdx.x & 31;
-    const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (y >= g.ny) return;  // uniform across the warp
-    const bool active = x0 < g.nx;
-    const Site<WALLS> s(active ? x0 : 0, y, z, 2, g);
+    const PairAt at(box, WALLS && !XONLY);
+    Site<WALLS> s(at.x0, at.y, at.z, 2, g);
+    drop_yz<XONLY>(s);
+    step_begin(box);
+    const int x0 = at.x0;
+    const bool active = at.active, head = at.head, last = at.last;
     R f0[Q], f1[Q];
-    gather2<true>(P, s, g, lane, active, f0, f1);
+    gather2<true>(P, s, at, f0, f1);
     if (active) {
         collide_lean<R, RHO0, one_rounding_v<T>>(f0, p);
         collide_lean<R, RHO0, one_rounding_v<T>>(f1, p);
     }
-    const bool last = lane == 31 || x0 + 2 >= g.nx;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int cx = CX(q);
@@ -446,7 +459,7 @@ __global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<ty
                 Pair<T>::store(bnc + s.own + x0, f0[q], f1[q]);
                 continue;
             }
-            if (lane == 0)
+            if (head)
                 Storage<T>::store(dst + trow + x0 + 1, f0[q]);
             else
                 Pair<T>::store(dst + trow + x0, left, f0[q]);
@@ -464,10 +477,11 @@ __global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<ty
                 Storage<T>::store(dst + trow + x0, f1[q]);
             else
                 Pair<T>::store(dst + trow + x0, f1[q], right);
-            if (lane == 0)  // cell x0 goes to x0 - 1: the previous segment, the periodic image, or a wall
+            if (head)  // cell x0 goes to x0 - 1: the previous segment, the periodic image, or a wall
                 Storage<T>::store((WALLS && s.bxm) ? bnc + s.own + x0 : dst + trow + s.xm, f0[q]);
         }
     }
+    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // ---------------------------------------------------------------- four cells per thread (16-bit storage)
@@ -629,6 +643,62 @@ __global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Pla
     step_begin(box);
     ab4_body<T, RHO0, WALLS, MRT>(src, dst, s, g, p);
     if constexpr (WALLS && !XONLY) step_end(box);
+}
+
+// A/B pull step for 16-bit storage whose rows hold pairs but not quads of cells
+// (nx even): the same windows, of two codes in a 32-bit word.
+// 190x131x97 FP16 42.8 -> 37.5 us against the shuffles of k_ab2, with walls on all
+// axes 62.8 -> 37.9; blocks per SM 5 / 6 / 8: 37.5 / 39.3 / 38.1 us, with walls
+// 39.6 / 37.9 / 44.2.
+template <typename T, bool RHO0, bool WALLS>
+__global__ void __launch_bounds__(128, WALLS ? 6 : 5) k_ab2w(Planes<T> src, Planes<T> dst, Geo g, Relax<float> p, Box box)
+{
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int xp, y, z;
+    box.at(i, xp, y, z);
+    const Site<WALLS> s(2 * xp, y, z, 2, g);
+    step_begin(box);
+    const int xprev = s.x == 0 ? g.nx - 2 : s.x - 2;
+    const int xnext = s.x + 2 >= g.nx ? 0 : s.x + 2;
+    unsigned win[Q], nb[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int cx = CX(q);
+        const bool w = s.template wall_yz<-1>(q);
+        const unsigned short *from = reinterpret_cast<const unsigned short *>(src.p[q]) + s.template row_along<-1>(q);
+        const unsigned short *own = reinterpret_cast<const unsigned short *>(src.p[OPP(q)]) + s.own + s.x;
+        win[q] = *reinterpret_cast<const unsigned *>(w ? own : from + s.x);
+        if (cx != 0) {
+            const bool xwall = WALLS && ((cx > 0 && s.bxm) || (cx < 0 && s.bxp));
+            nb[q] = *reinterpret_cast<const unsigned *>(xwall ? own : from + (cx > 0 ? xprev : xnext));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int cx = CX(q);
+        if (cx == 0 || s.template wall_yz<-1>(q)) continue;
+        if (cx > 0)  // [x0 - 1, x0]: element 1 of the pair before (or the reflected x0)
+            win[q] = __funnelshift_l(WALLS && s.bxm ? nb[q] << 16 : nb[q], win[q], 16);
+        else         // [x0 + 1, x0 + 2]: element 0 of the pair after (or the reflected x0 + 1)
+            win[q] = __funnelshift_r(win[q], WALLS && s.bxp ? nb[q] >> 16 : nb[q], 16);
+    }
+    float f[Q];
+    unsigned low[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) f[q] = Bits16<T>::to_float(win[q] & 0xffffu);
+    collide_lean<float, RHO0, false>(f, p);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        low[q] = Bits16<T>::from_float(f[q]);
+        f[q] = Bits16<T>::to_float(win[q] >> 16);
+        win[q] = low[q];
+    }
+    collide_lean<float, RHO0, false>(f, p);
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        *reinterpret_cast<unsigned *>(reinterpret_cast<unsigned short *>(dst.p[q]) + s.own + s.x) =
+            (Bits16<T>::from_float(f[q]) << 16) | (win[q] & 0xffffu);
 }
 
 // AA even step for 16-bit storage, four cells per thread: own quads of plane
@@ -949,14 +1019,23 @@ static cudaError_t step_t(int kind, void *src, void *dst, const Geo &g, const Co
         }
     }
     if (!cb.mrt && ls.cells_x >= 2 && (g.nx % 2) == 0 && (ls.bx % 32) == 0) {
-        const dim3 block(ls.bx, ls.by, 1);
-        const dim3 grid((g.nx + 2 * ls.bx - 1) / (2 * ls.bx), (g.ny + ls.by - 1) / ls.by, g.nz);
-        if (kind == 0)
-            k_ab2<T, RHO0, WALLS><<<grid, block, 0, stream>>>(planes_of<T>(src, g.ncell), D, g, p);
+        const Box box(g.nx / 2, 0, g.ny, 0, g.nz);
+        if (kind == 0) {
+            if constexpr (sizeof(T) == 2)
+                launch_step_box(k_ab2w<T, RHO0, WALLS>, true, box, 0, QUAD_THREADS, stream, planes_of<T>(src, g.ncell), D,
+                                g, p);
+            else
+                launch_step_box(k_ab2<T, RHO0, WALLS>, true, box, 0, threads, stream, planes_of<T>(src, g.ncell), D, g, p);
+        }
         else if (kind == 1)
-            k_aa_even2<T, RHO0><<<grid, block, 0, stream>>>(D, g, p);
+            launch_step_box(k_aa_even2<T, RHO0>, true, box, 0, threads, stream, D, g, p);
         else
-            k_aa_odd2<T, RHO0, WALLS><<<grid, block, 0, stream>>>(D, g, p);
+            split_rows<WALLS>(g, g.nx / 2, [&](int rows, const Box &part) {
+                auto k = rows == ROWS_WALLED   ? k_aa_odd2<T, RHO0, true>
+                         : rows == ROWS_XWALLS ? k_aa_odd2<T, RHO0, true, true>
+                                               : k_aa_odd2<T, RHO0, false>;
+                launch_step_box(k, true, part, 0, threads, stream, D, g, p);
+            });
         return cudaGetLastError();
     }
     if (cb.mrt)

@@ -69,3 +69,22 @@ def test_adjoint_of_any_row_length_matches_oracle(shape, walls):
     got = np.moveaxis(out.cpu().numpy()[perm], 0, -1)
     assert np.abs(got - lam_o).max() < 1e-12
     assert np.abs(gw.cpu().numpy() - g_o).max() < 1e-11 * nx * ny * nz
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 5), (6, 1, 2), (62, 5, 3), (66, 3, 4), (130, 2, 3), (254, 1, 1)])
+@pytest.mark.parametrize("precision", ["f16s", "bf16s"])
+@pytest.mark.parametrize("pattern", ["ab", "aa"])
+@pytest.mark.parametrize("walls", [(0, 0, 0), (0, 1, 0), (0, 0, 1), (1, 0, 0), (1, 1, 1)])
+def test_rows_of_pairs_match_one_cell_per_thread(shape, precision, pattern, walls):
+    """16-bit rows that hold pairs but no quads of cells: bitwise the one-cell kernels' populations."""
+    from paper_1803_04937_gb300.lbm import Simulation
+    nx, ny, nz = shape
+    rho, u = random_fields((nz, ny, nx), seed=nx + ny)
+    out = []
+    for cells_x in (4, 1):
+        sim = Simulation(nx, ny, nz, precision=precision, pattern=pattern, walls=walls, collision="trt", tau=0.7,
+                         force=(1e-4, -5e-5, 2e-5), cells_x=cells_x)
+        sim.init(rho.cuda(), u.cuda())
+        sim.step(5)
+        out.append(sim.get_pdfs())
+    assert torch.equal(out[0], out[1])
