@@ -5,9 +5,9 @@ fraction of the measured HBM roofline.
 Default workload: periodic 256^3 lattice, FP32 storage, SRT, D3Q19-I
 (improved) equilibrium, tau = 0.8, transverse shear wave u_y = 0.01 sin(2 pi
 x / 256) on a background flow U_x = 0.1.  A bench "step" is one lattice time
-step over all 256^3 cells (one launch of the fused stream + collide kernel).
-The 2 x 1.27 GB of population grids are ~20x the 129 MB L2, so every step
-streams from HBM (no L2 flush needed).
+step over all 256^3 cells; one launch of the fused stream + collide kernel
+computes one or (FP32 A/B) two of them.  The 2 x 1.27 GB of population grids are
+~20x the 129 MB L2, so every launch streams from HBM (no L2 flush needed).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl native|reference]
 
@@ -167,7 +167,7 @@ def read_traffic(kernel_key):
     if not e:
         return None, None
     src = b""
-    for f in ("lbm_device.cuh", "lbm_step.cuh"):
+    for f in ("lbm_device.cuh", "lbm_step.cuh", "lbm_pair.cuh"):
         src += open(os.path.join(ROOT, "paper_1803_04937_gb300", "csrc", f), "rb").read()
     sha = hashlib.sha256(src).hexdigest()[:16]
     if e.get("source_sha") != sha:
@@ -186,6 +186,18 @@ def measured_peaks():
 def shear_workload(nx, ny, nz, device):
     from paper_1803_04937_gb300 import inputs
     return inputs.shear_wave(nx, ny, nz, U=(0.1, 0.0, 0.0), amplitude=0.01, device=device)
+
+
+def steps_per_pass(args, n):
+    """Steps that one pass of the main workload's kernel over the grids computes: the library runs FP32 A/B
+    steps of larger periodic lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or cells per thread are set."""
+    pairs = args.precision == "f32" and args.pattern == "ab" and n >= 128 and not args.block and args.cells_x is None
+    return 2 if pairs else 1
+
+
+def step_launches(args, n, steps):
+    """Step kernels that lbm_step(steps) launches: pairs in groups of two, single steps for the rest."""
+    return steps if steps_per_pass(args, n) == 1 else steps // 4 * 2 + steps % 4
 
 
 # ------------------------------------------------------------------ GPU timing
@@ -515,12 +527,16 @@ def run_native(args):
     value = ws * cells * args.steps / t / 1e6
     per_launch = t_local / args.steps
     peak, peak_kind = measured_peaks()
-    achieved = BYTES_PER_LUP[args.precision] * cells / per_launch / 1e9
+    passes = steps_per_pass(args, n)
+    bytes_per_lup = BYTES_PER_LUP[args.precision] / passes  # every population read and written once per pass
+    achieved = bytes_per_lup * cells / per_launch / 1e9
     cx = args.cells_x or (4 if args.precision in ("f16s", "bf16s") else 1)
     if args.pattern == "ab":
         kname = "k_ab%d<%s>" % (cx, args.precision) + ("[mrt]" if args.collision == "mrt" else "")
     else:
         kname = "k_aa_even%d+k_aa_odd%d<%s>" % (cx, cx, args.precision) + ("[mrt]" if args.collision == "mrt" else "")
+    if passes == 2:
+        kname = "k_pair<f32>" + ("[mrt]" if args.collision == "mrt" else "")
     traffic_per_lup, _ = read_traffic(kname)
     line = {
         "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": ws, "steps": args.steps,
@@ -533,13 +549,13 @@ def run_native(args):
                    "l2": "inputs larger than L2 (%.2f GB per grid vs 129 MB L2)" % (
                        BYTES_PER_LUP[args.precision] / 2 * cells / 1e9),
                    "parallelism": "replicas x%d" % ws, "finite": ok},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+        "roofline": {"bound": "hbm" if passes == 1 else "issue", "steps_per_pass": passes, "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": peak_kind,
                      "peak_nominal": NOMINAL_HBM_GBS, "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
-                     "algorithmic_bytes_per_lup": BYTES_PER_LUP[args.precision],
+                     "algorithmic_bytes_per_lup": bytes_per_lup,
                      "traffic": traffic_per_lup * cells if traffic_per_lup else None,
                      "kernel": kname},
-        "gpu_launches": args.steps,
+        "gpu_launches": step_launches(args, n, args.steps),
         "clocks": sampler.summary(),
     }
     if not args.no_extras and ws > 1:

@@ -26,6 +26,7 @@ struct lbm_ctx {
     int bx = 128, by = 2;
     bool block_set = false;  // the caller chose bx or by
     int cells_x = 1;
+    int pairs = 1;                                 // two steps per pass: 0 never, 1 where it pays, 2 always
     int graphs = 1;                                // replay GRAPH_STEPS-step CUDA graphs in lbm_step
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // by starting A/B grid or AA parity
     void *a = nullptr, *b = nullptr;
@@ -226,6 +227,38 @@ cudaError_t launch_one(const lbm_ctx *h, cudaStream_t st, int &cur, int &parity,
     return e;
 }
 
+// Whether steps of this handle may run in pairs (launch_pair_f32).
+bool use_pairs(const lbm_ctx *h, const lbm::Geo &g)
+{
+    if (h->pairs == 0 || h->pattern != LBM_PATTERN_AB || h->precision != LBM_F32 || h->cells_x != 1 || h->block_set)
+        return false;
+    if (h->stencil != LBM_D3Q19) return false;
+    return h->pairs == 2 || lbm::pair_pays_f32(g);
+}
+
+// n time steps on stream st, advancing the A/B grid `cur` or AA parity
+// `parity`; done counts the steps that were enqueued.  Steps go in groups of
+// two pairs, so that n steps leave the state in the grid that n one-step
+// launches would leave it in.
+cudaError_t launch_steps(const lbm_ctx *h, cudaStream_t st, int &cur, int &parity, int n, int &done, const lbm::Geo &g,
+                         const lbm::CollBoth &c, const lbm::LaunchShape &shape)
+{
+    done = 0;
+    if (n >= 4 && use_pairs(h, g)) {
+        void *const from = cur ? h->b : h->a, *const to = cur ? h->a : h->b;
+        for (; done + 4 <= n; done += 4) {
+            cudaError_t e = lbm::launch_pair_f32(from, to, g, c, st);
+            if (e == cudaSuccess) e = lbm::launch_pair_f32(to, from, g, c, st);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    for (; done < n; ++done) {
+        cudaError_t e = launch_one(h, st, cur, parity, g, c, shape);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Steps per CUDA graph: even, so that a replay returns to the grid (A/B) or
 // parity (AA) it started from.
 constexpr int GRAPH_STEPS = 16;
@@ -249,9 +282,8 @@ cudaError_t build_graph(lbm_ctx *h, int slot, const lbm::Geo &g, const lbm::Coll
     if (e != cudaSuccess) return e;
     e = cudaStreamBeginCapture(ps, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        int cur = slot, parity = slot;
-        cudaError_t le = cudaSuccess;
-        for (int k = 0; k < GRAPH_STEPS && le == cudaSuccess; ++k) le = launch_one(h, ps, cur, parity, g, c, shape);
+        int cur = slot, parity = slot, done = 0;
+        const cudaError_t le = launch_steps(h, ps, cur, parity, GRAPH_STEPS, done, g, c, shape);
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(ps, &graph);
         if (le != cudaSuccess) e = le;
@@ -405,6 +437,10 @@ int lbm_set_option(lbm_handle h, int key, double v)
         if (v != 0.0 && v != 1.0) return fail(h, LBM_EINVAL, "graphs option must be 0 or 1");
         h->graphs = (int)v;
         return LBM_OK;
+    case LBM_OPT_STEP_PAIRS:
+        if (v != 0.0 && v != 1.0 && v != 2.0) return fail(h, LBM_EINVAL, "step pairs option must be 0, 1 or 2");
+        h->pairs = (int)v;
+        return LBM_OK;
     case LBM_OPT_ADJ_DEFER_SUM: {
         if (v != 0.0 && v != 1.0) return fail(h, LBM_EINVAL, "deferred adjoint sums option must be 0 or 1");
         const int st = adj_flush(h, "lbm_set_option (adjoint flush)");
@@ -450,6 +486,7 @@ int lbm_get_option(lbm_handle h, int key, double *v)
     case LBM_OPT_MRT_OMEGA_4: *v = h->omega_4; return LBM_OK;
     case LBM_OPT_CELLS_X: *v = h->cells_x; return LBM_OK;
     case LBM_OPT_GRAPHS: *v = h->graphs; return LBM_OK;
+    case LBM_OPT_STEP_PAIRS: *v = h->pairs; return LBM_OK;
     case LBM_OPT_ADJ_DEFER_SUM: *v = h->adj_defer; return LBM_OK;
     case LBM_OPT_BLOCK_X: *v = h->bx; return LBM_OK;
     case LBM_OPT_BLOCK_Y: *v = h->by; return LBM_OK;
@@ -540,11 +577,10 @@ int lbm_step(lbm_handle h, int n)
             }
         }
     }
-    for (; i < n; ++i) {
-        cudaError_t e = launch_one(h, h->stream, h->cur, h->parity, g, c, shape);
-        if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step");
-        ++h->t;
-    }
+    int done = 0;
+    const cudaError_t e = launch_steps(h, h->stream, h->cur, h->parity, n - i, done, g, c, shape);
+    h->t += done;
+    if (e != cudaSuccess) return cuda_fail(h, e, "lbm_step");
     return LBM_OK;
 }
 

@@ -873,11 +873,12 @@ static inline unsigned blocks_for(long long items, int threads) { return (unsign
 // already followed the end of the step before.
 template <typename... P, typename... A>
 static void launch_step_kernel(void (*kernel)(P...), bool early, dim3 grid, dim3 threads, cudaStream_t stream,
-                               A &&...args)
+                               int shared_bytes, A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = threads;
+    cfg.dynamicSmemBytes = (size_t)shared_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -894,12 +895,12 @@ static void launch_step_box(void (*kernel)(P...), bool early, const Box &box, in
                             A &&...args)
 {
     if (bx == 0) {
-        launch_step_kernel(kernel, early, blocks_for(box.count, threads), threads, stream, std::forward<A>(args)..., box);
+        launch_step_kernel(kernel, early, blocks_for(box.count, threads), threads, stream, 0, std::forward<A>(args)..., box);
         return;
     }
     const unsigned ux = (unsigned)bx, uy = (unsigned)(threads / bx);
     launch_step_kernel(kernel, early, dim3((box.per_row.d + ux - 1) / ux, (box.rows.d + uy - 1) / uy, (unsigned)box.nz),
-                       dim3(ux, uy), stream, std::forward<A>(args)..., box);
+                       dim3(ux, uy), stream, 0, std::forward<A>(args)..., box);
 }
 
 // The one-cell A/B step stays one launch over all rows: its walled kernel
@@ -981,7 +982,7 @@ static void launch_step1(int kind, void *src, const Planes<T> &D, const Geo &g,
     if (kind == 0)
         launch_ab1<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, threads, stream);
     else if (kind == 1)
-        launch_step_kernel(k_aa_even1<T, RHO0, MRT>, aa1_early<T>, blocks_for(g.ncell, threads), threads, stream, D, D, g, p,
+        launch_step_kernel(k_aa_even1<T, RHO0, MRT>, aa1_early<T>, blocks_for(g.ncell, threads), threads, stream, 0, D, D, g, p,
                            Box());
     else
         launch_aa_odd1<T, RHO0, WALLS, MRT>(D, g, p, threads, stream);
@@ -995,8 +996,8 @@ static void launch_step4(int kind, void *src, const Planes<T> &D, const Geo &g, 
     if (kind == 0)
         launch_ab4<T, RHO0, WALLS, MRT>(planes_of<T>(src, g.ncell), D, g, p, stream);
     else if (kind == 1)
-        launch_step_kernel(k_aa_even4<T, RHO0, MRT>, true, blocks_for(g.ncell / 4, QUAD_THREADS), QUAD_THREADS, stream, D,
-                           D, g, p, Box());
+        launch_step_kernel(k_aa_even4<T, RHO0, MRT>, true, blocks_for(g.ncell / 4, QUAD_THREADS), QUAD_THREADS, stream, 0,
+                           D, D, g, p, Box());
     else
         launch_aa_odd4<T, RHO0, WALLS, MRT>(D, g, p, stream);
 }
