@@ -6,7 +6,7 @@ Forward: f(0) = feq(rho, u0) (Eq. 14 or Eq. 22), T steps of Eq. 15 (A/B
 pattern), output (rho(T), u(T)) of Eq. 16-17.  Every ceil(sqrt(T)) steps the
 raw A/B grid is copied into a checkpoint.  Backward: lambda(T) from dL/du(T)
 and dL/drho(T); then, segment by segment from the last, the states of the
-segment are recomputed from its checkpoint into a ring of grids and the
+segment are recomputed from its checkpoint into a list of grids and the
 adjoint steps run in reverse; finally dL/du0 through f(0) = feq(rho, u0) and
 dL/dtau from the FP64 accumulators of dL/domega+-.  Memory: ~2 sqrt(T) grids.
 Supports rho0 = 1 (the paper's choice) only.
@@ -70,17 +70,17 @@ class _Run(torch.autograd.Function):
         check(lib.lbm_set_option(h, _lib.OPT_ADJ_DEFER_SUM, 1.0), h)
         check(lib.lbm_adjoint_seed(h, _ptr(grad_rho), _ptr(grad_u), dt, _ptr(lam[0])), h)
         cur = 0
-        ring = [torch.empty(shape, dtype=sim.storage_dtype, device=dev) for _ in range(min(every, nsteps) + 1)]
+        ring = [torch.empty(shape, dtype=sim.storage_dtype, device=dev) for _ in range(min(every, nsteps) - 1)]
         nseg = len(ctx.ckpts)
         for s in range(nseg - 1, -1, -1):
             t0 = s * every
             t1 = min(t0 + every, nsteps)
-            ring[0].copy_(ctx.ckpts[s])
+            states = [ctx.ckpts[s]] + ring  # the checkpoint is read in place
             for i in range(1, t1 - t0):  # states t0+1 .. t1-1
-                sim._bind(ring[i - 1], ring[i])
+                sim._bind(states[i - 1], states[i])
                 sim.step(1)
             for t in range(t1 - 1, t0 - 1, -1):
-                check(lib.lbm_adjoint_step(h, _ptr(ring[t - t0]), _ptr(lam[cur]), _ptr(lam[1 - cur]), _dp(gw)), h)
+                check(lib.lbm_adjoint_step(h, _ptr(states[t - t0]), _ptr(lam[cur]), _ptr(lam[1 - cur]), _dp(gw)), h)
                 cur = 1 - cur
         grad_u0 = torch.empty_like(u0)
         check(lib.lbm_adjoint_init_velocity(h, _ptr(rho) if rho.numel() else None, _ptr(u0), _field_dtype(u0),
