@@ -188,10 +188,11 @@ def shear_workload(nx, ny, nz, device):
     return inputs.shear_wave(nx, ny, nz, U=(0.1, 0.0, 0.0), amplitude=0.01, device=device)
 
 
-def steps_per_pass(args, n):
-    """Steps that one pass of the main workload's kernel over the grids computes: the library runs FP32 A/B
-    steps of larger periodic lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or cells per thread are set."""
-    pairs = args.precision == "f32" and args.pattern == "ab" and n >= 128 and not args.block and args.cells_x is None
+def steps_per_pass(args, n, precision=None, pattern=None, stencil=19, **_):
+    """Steps that one pass over the grids computes on a periodic n^3 lattice: the library runs FP32 A/B steps
+    of larger lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or cells per thread are set."""
+    pairs = (precision or args.precision) == "f32" and (pattern or args.pattern) == "ab" and not args.block and \
+        args.cells_x is None and n >= (128 if stencil == 19 else 160)
     return 2 if pairs else 1
 
 
@@ -248,7 +249,7 @@ def variant_mlups(args, n, **kw):
     sim = make_sim(args, n, **kw)
     t = time_steps(sim, 400, 10)
     prec = kw.get("precision") or args.precision
-    bpl = BYTES_PER_LUP[prec] * kw.get("stencil", 19) // 19
+    bpl = BYTES_PER_LUP[prec] * kw.get("stencil", 19) // 19 / steps_per_pass(args, n, **kw)
     out = {"mlups": n ** 3 / t / 1e6, "gbs": bpl * n ** 3 / t / 1e9}
     sim.close()
     del sim
@@ -278,7 +279,8 @@ def config_variants(peak):
         t = time_steps(sim, 200, 10)
         cells = 512 * 256 * 256
         key = "channel_512x256x256_" + prec + ("" if pattern == "ab" else "_aa")
-        out[key] = {"mlups": cells / t / 1e6, "gbs": BYTES_PER_LUP[prec] * cells / t / 1e9,
+        passes = 2 if (prec, pattern) == ("f32", "ab") else 1  # steps in pairs
+        out[key] = {"mlups": cells / t / 1e6, "gbs": BYTES_PER_LUP[prec] / passes * cells / t / 1e9,
                     "profile_err_after_5000_steps": CHANNEL_PROFILE_ERR[prec]}
         sim.close()
         del sim

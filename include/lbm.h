@@ -124,7 +124,7 @@ typedef struct lbm_ctx *lbm_handle;
                                  Same results either way. */
 #define LBM_OPT_STEP_PAIRS 20 /* 1 (default): lbm_step computes two time steps per pass over the
                                  grids (the state between them stays on the chip) where that is
-                                 faster: D3Q19, A/B pattern, FP32 storage, larger lattices, no
+                                 faster: A/B pattern, FP32 storage, larger lattices, no
                                  LBM_OPT_CELLS_X or LBM_OPT_BLOCK_* chosen; 0: never; 2: for
                                  every such lattice.  The same populations either way, in the
                                  same grid; the grid that does not hold the current state then

@@ -232,8 +232,7 @@ bool use_pairs(const lbm_ctx *h, const lbm::Geo &g)
 {
     if (h->pairs == 0 || h->pattern != LBM_PATTERN_AB || h->precision != LBM_F32 || h->cells_x != 1 || h->block_set)
         return false;
-    if (h->stencil != LBM_D3Q19) return false;
-    return h->pairs == 2 || lbm::pair_pays_f32(g);
+    return h->pairs == 2 || (h->stencil == LBM_D3Q27 ? lbm::pair_pays27_f32(g) : lbm::pair_pays_f32(g));
 }
 
 // n time steps on stream st, advancing the A/B grid `cur` or AA parity
@@ -246,9 +245,10 @@ cudaError_t launch_steps(const lbm_ctx *h, cudaStream_t st, int &cur, int &parit
     done = 0;
     if (n >= 4 && use_pairs(h, g)) {
         void *const from = cur ? h->b : h->a, *const to = cur ? h->a : h->b;
+        const auto pair = h->stencil == LBM_D3Q27 ? lbm::launch_pair27_f32 : lbm::launch_pair_f32;
         for (; done + 4 <= n; done += 4) {
-            cudaError_t e = lbm::launch_pair_f32(from, to, g, c, st);
-            if (e == cudaSuccess) e = lbm::launch_pair_f32(to, from, g, c, st);
+            cudaError_t e = pair(from, to, g, c, st);
+            if (e == cudaSuccess) e = pair(to, from, g, c, st);
             if (e != cudaSuccess) return e;
         }
     }

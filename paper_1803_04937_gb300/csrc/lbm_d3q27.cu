@@ -9,6 +9,7 @@
 // D3Q27 lattices.  (Reductions, AA and the adjoint are D3Q19 only.)
 #include <cmath>
 
+#include "lbm_pair.cuh"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -298,6 +299,24 @@ __global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g,
     if constexpr (WALLS && !XONLY) step_end(box);
 }
 
+// The lattice for two FP32 steps per pass (k_pair).  16 rows leave 128 registers a
+// thread for the 27 populations in hand and the 27 on their way; with 20 rows they
+// spill (256^3: 454 against 564 us a step, one-step kernel 520; walled channel
+// 512x256x256 954 against 1567, one-step 1067).
+struct Lat27 {
+    static constexpr int NQ = Q27;
+    using Consts = Relax27<float>;
+    template <bool WALLS> static constexpr int warps = 16;
+    static __host__ __device__ constexpr int cx(int q) { return CX(q); }
+    static __host__ __device__ constexpr int cy(int q) { return CY(q); }
+    static __host__ __device__ constexpr int cz(int q) { return CZ(q); }
+    template <bool RHO0, bool WALLS, bool MRT>
+    static __device__ __forceinline__ void collide(float g[Q27], const Relax27<float> &p)
+    {
+        collide27<float, RHO0, true>(g, p);
+    }
+};
+
 // Writes the canonical populations fc (f_q(x) - w_q) of cell x into an A/B
 // grid so that the pull gather returns them: plane q at x - c_q, or through a
 // wall plane qbar of x.
@@ -489,6 +508,19 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
         launch_step_box(k, true, box, bx, s.threads, stream, a, b, g, p);
         return cudaGetLastError();
     });
+}
+
+bool pair_pays27_f32(const Geo &g) { return pair_pays<q27::Lat27>(g, 3.05, 3.25, 32.0); }
+
+cudaError_t launch_pair27_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t s)
+{
+    using L = q27::Lat27;
+    const q27::Relax27<float> p = q27::to_relax27<float>(c);
+    const PairPlanes<L> S = pair_planes<L>(src, g.ncell), D = pair_planes<L>(dst, g.ncell);
+    const bool walls = g.wall_x || g.wall_y || g.wall_z;
+    if (c.rho0_is_rho)
+        return walls ? launch_pair_k<L, true, true, false>(S, D, g, p, s) : launch_pair_k<L, true, false, false>(S, D, g, p, s);
+    return walls ? launch_pair_k<L, false, true, false>(S, D, g, p, s) : launch_pair_k<L, false, false, false>(S, D, g, p, s);
 }
 
 cudaError_t launch_init27(int prec, void *grid, const void *rho, const void *u, int dtype, const Geo &g,

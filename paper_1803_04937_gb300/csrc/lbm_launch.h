@@ -32,10 +32,12 @@ struct CollBoth {
 cudaError_t launch_step(int prec, int kind, const void *src, void *dst, const Geo &g, const CollBoth &c,
                         LaunchShape s, cudaStream_t stream);
 
-// Two A/B steps in one pass (src -> dst), D3Q19, FP32 storage; pair_pays_f32: whether
-// they are faster than two one-step launches on this lattice.
+// Two A/B steps in one pass (src -> dst), FP32 storage, D3Q19 and D3Q27; pair_pays:
+// whether they are faster than two one-step launches on this lattice.
 bool pair_pays_f32(const Geo &g);
 cudaError_t launch_pair_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);
+bool pair_pays27_f32(const Geo &g);
+cudaError_t launch_pair27_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);
 
 // f = feq(rho, u) written into `grid` for layout (0: AB, 1: AA even).
 cudaError_t launch_init(int prec, int layout, void *grid, const void *rho, const void *u, int dtype,

@@ -155,6 +155,9 @@ __device__ __forceinline__ void collide_packed(float g[Q], const RelaxPacked &p)
 
 struct Lat19 {
     static constexpr int NQ = Q;
+    using Consts = RelaxPacked;
+    // 24 rows leave 80 registers a thread, 20 leave 96, which the wall logic needs
+    template <bool WALLS> static constexpr int warps = WALLS ? 20 : 24;
     static __host__ __device__ constexpr int cx(int q) { return CX(q); }
     static __host__ __device__ constexpr int cy(int q) { return CY(q); }
     static __host__ __device__ constexpr int cz(int q) { return CZ(q); }
@@ -188,13 +191,12 @@ struct PairRing {
     }
 };
 
-// Rows of a tile in step 1, one warp each: 24 leave 80 registers a thread, 20
-// leave 96, which the wall logic needs.
-template <bool WALLS> constexpr int pair_warps = WALLS ? 20 : 24;
+// Rows of a tile in step 1, one warp each.
+template <typename L, bool WALLS> constexpr int pair_warps = L::template warps<WALLS>;
 
 template <typename L, bool WALLS> constexpr int pair_smem()
 {
-    return PairRing<L, WALLS>::SLOTS * (pair_warps<WALLS> - 2) * PAIR_LANES * 4;
+    return PairRing<L, WALLS>::SLOTS * (pair_warps<L, WALLS> - 2) * PAIR_LANES * 4;
 }
 
 struct PairTiles {
@@ -207,12 +209,12 @@ template <typename L> struct PairPlanes {
 };
 
 template <typename L, bool RHO0, bool WALLS, bool MRT>
-__global__ void __launch_bounds__(pair_warps<WALLS> *PAIR_LANES, 1)
-    k_pair(PairPlanes<L> src, PairPlanes<L> dst, Geo g, RelaxPacked p, PairTiles t)
+__global__ void __launch_bounds__(pair_warps<L, WALLS> *PAIR_LANES, 1)
+    k_pair(PairPlanes<L> src, PairPlanes<L> dst, Geo g, typename L::Consts p, PairTiles t)
 {
     using Ring = PairRing<L, WALLS>;
     constexpr int NQ = L::NQ;
-    constexpr int W = pair_warps<WALLS>;
+    constexpr int W = pair_warps<L, WALLS>;
     constexpr int COLS = (W - 2) * PAIR_LANES;
     extern __shared__ float sh[];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
@@ -348,24 +350,26 @@ static inline PairTiles pair_tiles(const Geo &g, int out_rows, dim3 &grid, long 
     return t;
 }
 
-// Whether two steps go through k_pair: where its iterations (2.7 to 2.95 us each,
-// with walls 2.4 to 2.7) take less time than two one-step launches, which run at 45.5 GLUPS
-// from DRAM.  Not with walls on x, whose ends put half of the warps on the wall
-// path (closed box 256x192x160: 172 against 210 us), for lattices whose grids stay in L2 (both below 200 MB; 96^3:
-// 20 us a step against 22), nor for more tile rows than a grid may have.
-static inline bool pair_pays(const Geo &g)
+// Whether two steps go through k_pair: where its iterations (D3Q19: 2.7 to 2.95 us
+// each, with walls 2.4 to 2.7) take less time than two one-step launches, which run
+// at `glups` from DRAM.  Not with walls on x, whose ends put half of the warps on
+// the wall path (closed box 256x192x160: 172 against 210 us), for lattices whose
+// grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22), nor for more
+// tile rows than a grid may have.
+template <typename L>
+static inline bool pair_pays(const Geo &g, double us_iteration, double us_iteration_walls, double glups)
 {
     const bool walls = g.wall_x || g.wall_y || g.wall_z;
     dim3 grid;
     long long iterations;
-    pair_tiles(g, (walls ? pair_warps<true> : pair_warps<false>) - 2, grid, iterations);
-    return !g.wall_x && g.ncell * 152 >= 200000000 && grid.y <= 65535 &&
-           iterations * (walls ? 2.7 : 2.8) < 2.0 * (double)g.ncell / 45.5e3;
+    pair_tiles(g, (walls ? pair_warps<L, true> : pair_warps<L, false>) - 2, grid, iterations);
+    return !g.wall_x && g.ncell * 8 * L::NQ >= 200000000 && grid.y <= 65535 &&
+           iterations * (walls ? us_iteration_walls : us_iteration) < 2.0 * (double)g.ncell / (glups * 1e3);
 }
 
 template <typename L, bool RHO0, bool WALLS, bool MRT>
 static cudaError_t launch_pair_k(const PairPlanes<L> &S, const PairPlanes<L> &D, const Geo &g,
-                                 const RelaxPacked &p, cudaStream_t stream)
+                                 const typename L::Consts &p, cudaStream_t stream)
 {
     constexpr int smem = pair_smem<L, WALLS>();
     static_assert(smem <= 227 * 1024, "tile does not fit shared memory");
@@ -374,8 +378,8 @@ static cudaError_t launch_pair_k(const PairPlanes<L> &S, const PairPlanes<L> &D,
     if (e != cudaSuccess) return e;
     dim3 grid;
     long long iterations;
-    const PairTiles t = pair_tiles(g, pair_warps<WALLS> - 2, grid, iterations);
-    launch_step_kernel(k, true, grid, pair_warps<WALLS> * PAIR_LANES, stream, smem, S, D, g, p, t);
+    const PairTiles t = pair_tiles(g, pair_warps<L, WALLS> - 2, grid, iterations);
+    launch_step_kernel(k, true, grid, pair_warps<L, WALLS> * PAIR_LANES, stream, smem, S, D, g, p, t);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,6 @@
 """Two steps per pass (LBM_OPT_STEP_PAIRS) give bitwise the populations of
 one-step launches, in the same grid, for lattices that end anywhere within a
-tile (30 x 22 columns, 30 x 18 with walls) or a block's planes."""
+tile (30 x 22 columns, 30 x 18 with walls; D3Q27 30 x 14) or a block's planes."""
 import pytest
 import torch
 
@@ -39,6 +39,18 @@ def test_pairs_are_bitwise_single_steps(shape, walls, collision, equilibrium, rh
     assert out[0][2] == out[1][2] == 9
 
 
+@pytest.mark.parametrize("shape", SHAPES + [(60, 28, 7), (31, 15, 9)])
+@pytest.mark.parametrize("walls", WALLS)
+@pytest.mark.parametrize("rho0", [False, True])
+def test_d3q27_pairs_are_bitwise_single_steps(shape, walls, rho0):
+    out = []
+    for pairs in (0, 2):
+        sim = _sim(shape, pairs, walls=walls, collision="trt", equilibrium="standard", rho0_is_rho=rho0, stencil=27)
+        sim.step(9)
+        out.append(sim.get_pdfs())
+    assert torch.equal(out[0], out[1])
+
+
 @pytest.mark.parametrize("n", [3, 4, 6, 16, 23])
 @pytest.mark.parametrize("graphs", [False, True])
 def test_any_number_of_steps(n, graphs):
@@ -71,7 +83,7 @@ def test_unsupported_forms_step_singly():
     from paper_1803_04937_gb300 import _lib
     from paper_1803_04937_gb300.lbm import Simulation
     for kw in (dict(precision="f64"), dict(precision="f16s"), dict(precision="f32", pattern="aa"),
-               dict(precision="f32", stencil=27), dict(precision="f32", cells_x=2)):
+               dict(precision="f32", cells_x=2), dict(precision="f32", block=(64, 2))):
         out = []
         for pairs in (0, 2):
             sim = Simulation(36, 20, 6, tau=0.8, **kw)
