@@ -403,40 +403,6 @@ __device__ __forceinline__ R rest_equilibrium(R uu, R drho, R rho0, R kappa)
     return WQ<R>(0) * (drho - rho0 * R(1.5) * uu) + kappa * rho0 * uu * (R(1) / R(6));
 }
 
-// Collision in place: g <- g - omega+ (g+ - geq+) - omega- (g- - geq-) +
-// (1 - omega-/2) F_q.  For SRT omega- = omega+ and this is Eq. 15.
-template <typename R, int k>
-__device__ __forceinline__ void collide_pair(R g[Q], const R u[3], R uu, R drho, R rho0, const Coll<R> &p)
-{
-    constexpr int q = 2 * k + 1;
-    R sym, asym;
-    pair_equilibrium<R, q>(u, uu, drho, rho0, p.kappa, sym, asym);
-    R gp = R(0.5) * (g[q] + g[q + 1]);
-    R gm = R(0.5) * (g[q] - g[q + 1]);
-    R a1 = p.omega_p * (gp - sym);
-    R a2 = p.omega_m * (gm - asym);
-    g[q] = g[q] - a1 - a2 + p.force[k];
-    g[q + 1] = g[q + 1] - a1 + a2 - p.force[k];
-}
-
-template <typename R>
-__device__ __forceinline__ void collide(R g[Q], const Coll<R> &p)
-{
-    R drho, rho0, u[3];
-    macro(g, p, drho, rho0, u);
-    R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    g[0] = g[0] - p.omega_p * (g[0] - rest_equilibrium(uu, drho, rho0, p.kappa));
-    collide_pair<R, 0>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 1>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 2>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 3>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 4>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 5>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 6>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 7>(g, u, uu, drho, rho0, p);
-    collide_pair<R, 8>(g, u, uu, drho, rho0, p);
-}
-
 // ---------------------------------------------------------------- lean collision (step kernels)
 
 // Products and fused multiply-adds of the collision, written out (plain

@@ -14,7 +14,8 @@
 // are formed once per thread.  WALLS = false compiles the periodic lattice
 // without any bounce-back logic.
 //
-// Three thread mappings:
+// Three thread mappings, each over the lattice as one sequence of cells, pairs or
+// quads (Box):
 //  - one cell per thread (any nx; the FP32 and FP64 default): scalar loads;
 //    the +-x populations are read one element off alignment, which L1/L2
 //    absorb without extra DRAM traffic.
@@ -22,7 +23,8 @@
 //    and written as an aligned pair (half2 / bfloat162 / float2 / double2);
 //    a +-x shifted pair is assembled from the own pair and one element of the
 //    neighbouring lane's pair (warp shuffle), with one scalar access at the
-//    warp's edge.
+//    ends of the warp's part of a row.  (16-bit A/B steps form it from two words
+//    by a funnel shift instead, k_ab2w.)
 //  - four cells per thread (16-bit storage, nx % 4 == 0; the 16-bit default):
 //    8-byte quads of raw 16-bit codes; a +-x shifted window is formed from the
 //    aligned quad and its aligned neighbour quad by funnel shifts (load4w).
@@ -617,12 +619,10 @@ __device__ __forceinline__ void ab4_body(const Planes<T> &src, const Planes<T> &
         *reinterpret_cast<uint2 *>(reinterpret_cast<unsigned short *>(dst.p[q]) + s.own + s.x) = win[q];
 }
 
-// Resident blocks per SM for k_ab4.  The walled FP16 kernel (both code paths
-// inlined) spills at five blocks and runs faster at four with no spills; the
-// walled BF16 kernel is the other way round (measured with the walled channel
-// 512x256x256 as one walled launch: FP16 82.9 -> 84.5 GLUPS at four, BF16
-// 79.9 -> 74.4).  With split_rows the walled kernel runs only the wall rows,
-// or whole lattices with walls on x.
+// Resident blocks per SM for k_ab4.  The walled kernel runs only the rows at y and
+// z walls (split_rows); over a whole walled lattice FP16 was faster at four blocks
+// and BF16 at five (walled channel 512x256x256: FP16 82.9 -> 84.5 GLUPS at four,
+// BF16 79.9 -> 74.4).
 template <typename T, bool WALLS>
 constexpr int ab4_blocks = (WALLS && std::is_same_v<T, __half>) ? 4 : 5;
 
