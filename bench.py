@@ -190,9 +190,9 @@ def shear_workload(nx, ny, nz, device):
 
 def steps_per_pass(args, n, precision=None, pattern=None, stencil=19, **_):
     """Steps that one pass over the grids computes on a periodic n^3 lattice: the library runs FP32 A/B steps
-    of larger lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or cells per thread are set."""
+    of larger lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or two cells per thread are set."""
     pairs = (precision or args.precision) == "f32" and (pattern or args.pattern) == "ab" and not args.block and \
-        args.cells_x is None and n >= (128 if stencil == 19 else 160)
+        args.cells_x in (None, 1) and n >= (128 if stencil == 19 else 160)
     return 2 if pairs else 1
 
 

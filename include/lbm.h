@@ -124,9 +124,9 @@ typedef struct lbm_ctx *lbm_handle;
                                  Same results either way. */
 #define LBM_OPT_STEP_PAIRS 20 /* 1 (default): lbm_step computes two time steps per pass over the
                                  grids (the state between them stays on the chip) where that is
-                                 faster: A/B pattern, FP32 storage, larger lattices, no
-                                 LBM_OPT_CELLS_X or LBM_OPT_BLOCK_* chosen; 0: never; 2: for
-                                 every such lattice.  The same populations either way, in the
+                                 faster: A/B pattern, FP32 storage, LBM_OPT_CELLS_X = 1, no
+                                 LBM_OPT_BLOCK_* set, larger lattices; 0: never; 2: for every
+                                 size of such a lattice.  The same populations either way, in the
                                  same grid; the grid that does not hold the current state then
                                  holds one that is two steps older, not one. */
 #define LBM_OPT_ADJ_DEFER_SUM 19  /* 0 (default): each lbm_adjoint_step adds its dL/domega
