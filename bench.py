@@ -188,17 +188,15 @@ def shear_workload(nx, ny, nz, device):
     return inputs.shear_wave(nx, ny, nz, U=(0.1, 0.0, 0.0), amplitude=0.01, device=device)
 
 
-def steps_per_pass(args, n, precision=None, pattern=None, stencil=19, **_):
-    """Steps that one pass over the grids computes on a periodic n^3 lattice: the library runs FP32 A/B steps
-    of larger lattices in pairs (LBM_OPT_STEP_PAIRS) unless a block or two cells per thread are set."""
-    pairs = (precision or args.precision) == "f32" and (pattern or args.pattern) == "ab" and not args.block and \
-        args.cells_x in (None, 1) and n >= (128 if stencil == 19 else 160)
-    return 2 if pairs else 1
+def steps_per_pass(sim):
+    """Steps that one pass over the grids of this simulation computes, as the library decides it."""
+    from paper_1803_04937_gb300 import _lib
+    return int(sim.option(_lib.OPT_STEPS_PER_PASS))
 
 
-def step_launches(args, n, steps):
+def step_launches(passes, steps):
     """Step kernels that lbm_step(steps) launches: pairs in groups of two, single steps for the rest."""
-    return steps if steps_per_pass(args, n) == 1 else steps // 4 * 2 + steps % 4
+    return steps if passes == 1 else steps // 4 * 2 + steps % 4
 
 
 # ------------------------------------------------------------------ GPU timing
@@ -249,7 +247,7 @@ def variant_mlups(args, n, **kw):
     sim = make_sim(args, n, **kw)
     t = time_steps(sim, 400, 10)
     prec = kw.get("precision") or args.precision
-    bpl = BYTES_PER_LUP[prec] * kw.get("stencil", 19) // 19 / steps_per_pass(args, n, **kw)
+    bpl = BYTES_PER_LUP[prec] * kw.get("stencil", 19) // 19 / steps_per_pass(sim)
     out = {"mlups": n ** 3 / t / 1e6, "gbs": bpl * n ** 3 / t / 1e9}
     sim.close()
     del sim
@@ -279,8 +277,7 @@ def config_variants(peak):
         t = time_steps(sim, 200, 10)
         cells = 512 * 256 * 256
         key = "channel_512x256x256_" + prec + ("" if pattern == "ab" else "_aa")
-        passes = 2 if (prec, pattern) == ("f32", "ab") else 1  # steps in pairs
-        out[key] = {"mlups": cells / t / 1e6, "gbs": BYTES_PER_LUP[prec] / passes * cells / t / 1e9,
+        out[key] = {"mlups": cells / t / 1e6, "gbs": BYTES_PER_LUP[prec] / steps_per_pass(sim) * cells / t / 1e9,
                     "profile_err_after_5000_steps": CHANNEL_PROFILE_ERR[prec]}
         sim.close()
         del sim
@@ -521,6 +518,7 @@ def run_native(args):
     t = max_over_ranks(t_local, dist, device)
     red = sim.reduce()
     ok = red["nonfinite"] == 0
+    passes = steps_per_pass(sim)
     sim.close()
     del sim
     torch.cuda.empty_cache()
@@ -529,7 +527,6 @@ def run_native(args):
     value = ws * cells * args.steps / t / 1e6
     per_launch = t_local / args.steps
     peak, peak_kind = measured_peaks()
-    passes = steps_per_pass(args, n)
     bytes_per_lup = BYTES_PER_LUP[args.precision] / passes  # every population read and written once per pass
     achieved = bytes_per_lup * cells / per_launch / 1e9
     cx = args.cells_x or (4 if args.precision in ("f16s", "bf16s") else 1)
@@ -557,7 +554,7 @@ def run_native(args):
                      "algorithmic_bytes_per_lup": bytes_per_lup,
                      "traffic": traffic_per_lup * cells if traffic_per_lup else None,
                      "kernel": kname},
-        "gpu_launches": step_launches(args, n, args.steps),
+        "gpu_launches": step_launches(passes, args.steps),
         "clocks": sampler.summary(),
     }
     if not args.no_extras and ws > 1:

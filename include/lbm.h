@@ -129,6 +129,9 @@ typedef struct lbm_ctx *lbm_handle;
                                  size of such a lattice.  The same populations either way, in the
                                  same grid; the grid that does not hold the current state then
                                  holds one that is two steps older, not one. */
+#define LBM_OPT_STEPS_PER_PASS 21 /* read only: 2 if lbm_step runs steps in pairs on this handle as
+                                 it is now (LBM_OPT_STEP_PAIRS; n >= 4 steps go in groups of two
+                                 pairs, the rest singly), 1 if it runs every step by itself */
 #define LBM_OPT_ADJ_DEFER_SUM 19  /* 0 (default): each lbm_adjoint_step adds its dL/domega
                                  terms to its grad_omega before the call's work ends; 1:
                                  the terms of a step are summed by the next lbm_adjoint_step

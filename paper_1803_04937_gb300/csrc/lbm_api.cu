@@ -441,6 +441,7 @@ int lbm_set_option(lbm_handle h, int key, double v)
         if (v != 0.0 && v != 1.0 && v != 2.0) return fail(h, LBM_EINVAL, "step pairs option must be 0, 1 or 2");
         h->pairs = (int)v;
         return LBM_OK;
+    case LBM_OPT_STEPS_PER_PASS: return fail(h, LBM_EINVAL, "LBM_OPT_STEPS_PER_PASS is read only");
     case LBM_OPT_ADJ_DEFER_SUM: {
         if (v != 0.0 && v != 1.0) return fail(h, LBM_EINVAL, "deferred adjoint sums option must be 0 or 1");
         const int st = adj_flush(h, "lbm_set_option (adjoint flush)");
@@ -487,6 +488,7 @@ int lbm_get_option(lbm_handle h, int key, double *v)
     case LBM_OPT_CELLS_X: *v = h->cells_x; return LBM_OK;
     case LBM_OPT_GRAPHS: *v = h->graphs; return LBM_OK;
     case LBM_OPT_STEP_PAIRS: *v = h->pairs; return LBM_OK;
+    case LBM_OPT_STEPS_PER_PASS: *v = use_pairs(h, geo(h)) ? 2 : 1; return LBM_OK;
     case LBM_OPT_ADJ_DEFER_SUM: *v = h->adj_defer; return LBM_OK;
     case LBM_OPT_BLOCK_X: *v = h->bx; return LBM_OK;
     case LBM_OPT_BLOCK_Y: *v = h->by; return LBM_OK;

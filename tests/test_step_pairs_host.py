@@ -1,0 +1,51 @@
+"""Host-side decision of running steps in pairs (LBM_OPT_STEPS_PER_PASS), without a GPU."""
+import ctypes
+import inspect
+
+import pytest
+
+import bench
+from paper_1803_04937_gb300 import _lib
+
+F32, F16S = _lib.F32, _lib.F16S
+
+
+class _Handle:
+    """A handle with options, as Simulation has them, without device memory."""
+
+    def __init__(self, shape, stencil=19, precision=F32, options=()):
+        self.lib = _lib.load(build_if_missing=True)
+        self.h = ctypes.c_void_p()
+        assert self.lib.lbm_create(*shape, stencil, 0, 0, 0.8, precision, ctypes.byref(self.h)) == 0
+        for key, value in options:
+            assert self.lib.lbm_set_option(self.h, key, float(value)) == 0
+
+    def __del__(self):
+        self.lib.lbm_destroy(self.h)
+
+    def option(self, key):
+        v = ctypes.c_double()
+        assert self.lib.lbm_get_option(self.h, key, ctypes.byref(v)) == 0
+        return v.value
+
+
+@pytest.mark.parametrize("n", [96, 110, 120, 127, 128, 256])
+def test_bench_states_the_librarys_decision(n):
+    sim = _Handle((n, n, n))
+    passes = bench.steps_per_pass(sim)
+    assert passes == sim.option(_lib.OPT_STEPS_PER_PASS) == (1 if n < 110 else 2)  # 2 x 76 n^3 bytes from 200 MB on
+    assert bench.step_launches(passes, 23) == (23 if passes == 1 else 5 * 2 + 3)
+    assert list(inspect.signature(bench.steps_per_pass).parameters) == ["sim"]  # no rule of its own
+
+
+@pytest.mark.parametrize("kw", [dict(precision=F16S), dict(options=[(_lib.OPT_PATTERN, _lib.PATTERN_AA)]),
+                                dict(options=[(_lib.OPT_CELLS_X, 2)]), dict(options=[(_lib.OPT_STEP_PAIRS, 0)]),
+                                dict(options=[(_lib.OPT_WALLS_X, 1)])])
+def test_forms_that_step_singly(kw):
+    assert _Handle((256, 256, 256), **kw).option(_lib.OPT_STEPS_PER_PASS) == 1
+
+
+def test_the_decision_is_read_only():
+    sim = _Handle((8, 8, 8))
+    assert sim.lib.lbm_set_option(sim.h, _lib.OPT_STEPS_PER_PASS, 2.0) == _lib.LBM_EINVAL
+    assert b"read only" in sim.lib.lbm_last_error(sim.h)
