@@ -126,7 +126,9 @@ typedef struct lbm_ctx *lbm_handle;
                                  grids (the state between them stays on the chip) where that is
                                  faster: A/B pattern, FP32 storage, LBM_OPT_CELLS_X = 1, no
                                  LBM_OPT_BLOCK_* set, larger lattices; 0: never; 2: for every
-                                 size of such a lattice.  The same populations either way, in the
+                                 size of such a lattice but those the kernel cannot address (nx ny
+                                 from 2^30 on, nx or ny above 2^29, or ny above about 900,000),
+                                 which step singly.  The same populations either way, in the
                                  same grid; the grid that does not hold the current state then
                                  holds one that is two steps older, not one. */
 #define LBM_OPT_STEPS_PER_PASS 21 /* read only: 2 if lbm_step runs steps in pairs on this handle as

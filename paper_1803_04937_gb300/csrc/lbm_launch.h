@@ -32,11 +32,12 @@ struct CollBoth {
 cudaError_t launch_step(int prec, int kind, const void *src, void *dst, const Geo &g, const CollBoth &c,
                         LaunchShape s, cudaStream_t stream);
 
-// Two A/B steps in one pass (src -> dst), FP32 storage, D3Q19 and D3Q27; pair_pays:
-// whether they are faster than two one-step launches on this lattice.
-bool pair_pays_f32(const Geo &g);
+// Two A/B steps in one pass (src -> dst), FP32 storage, D3Q19 and D3Q27; pair_runs:
+// whether they can run on this lattice and (unless always) are faster than two
+// one-step launches.
+bool pair_runs_f32(const Geo &g, bool always);
 cudaError_t launch_pair_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);
-bool pair_pays27_f32(const Geo &g);
+bool pair_runs27_f32(const Geo &g, bool always);
 cudaError_t launch_pair27_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);
 
 // f = feq(rho, u) written into `grid` for layout (0: AB, 1: AA even).

@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(pair_warps<L, WALLS> *PAIR_LANES, 1)
     const bool in1 = lane <= wx + 1 && row <= wy + 1 && !(WALLS && g.wall_x && (xr < 0 || xr >= g.nx)) &&
                      !(WALLS && g.wall_y && (yr < 0 || yr >= g.ny));
     const bool in2 = lane >= 1 && lane <= wx && row >= 1 && row <= wy;
-    // wrapped columns and rows around the cell, in bytes (any offset a thread forms is in range)
+    // wrapped columns and rows around the cell, in bytes (any offset a thread forms is in range, see pair_runs)
     unsigned xs[3], ys[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -350,21 +350,25 @@ static inline PairTiles pair_tiles(const Geo &g, int out_rows, dim3 &grid, long 
     return t;
 }
 
-// Whether two steps go through k_pair: where its iterations (D3Q19: 2.7 to 2.95 us
+// Whether two steps go through k_pair.  It addresses a plane by 32-bit byte offsets
+// and forms wrapped coordinates as int, up to three edges long: a plane of 2^30 cells or
+// more, an edge above 2^29, or more tile rows than a grid may have are stepped singly
+// whatever is asked (`always`).  Otherwise where its iterations (D3Q19: 2.7 to 2.95 us
 // each, with walls 2.4 to 2.7) take less time than two one-step launches, which run
 // at `glups` from DRAM.  Not with walls on x, whose ends put half of the warps on
-// the wall path (closed box 256x192x160: 172 against 210 us), for lattices whose
-// grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22), nor for more
-// tile rows than a grid may have.
+// the wall path (closed box 256x192x160: 172 against 210 us), nor for lattices whose
+// grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22).
 template <typename L>
-static inline bool pair_pays(const Geo &g, double us_iteration, double us_iteration_walls, double glups)
+static inline bool pair_runs(const Geo &g, bool always, double us_iteration, double us_iteration_walls, double glups)
 {
+    if ((long long)g.nx * g.ny >= 1LL << 30 || g.nx > 1 << 29 || g.ny > 1 << 29) return false;
     const bool walls = g.wall_x || g.wall_y || g.wall_z;
     dim3 grid;
     long long iterations;
     pair_tiles(g, (walls ? pair_warps<L, true> : pair_warps<L, false>) - 2, grid, iterations);
-    return !g.wall_x && g.ncell * 8 * L::NQ >= 200000000 && grid.y <= 65535 &&
-           iterations * (walls ? us_iteration_walls : us_iteration) < 2.0 * (double)g.ncell / (glups * 1e3);
+    if (grid.y > 65535) return false;
+    return always || (!g.wall_x && g.ncell * 8 * L::NQ >= 200000000 &&
+                      iterations * (walls ? us_iteration_walls : us_iteration) < 2.0 * (double)g.ncell / (glups * 1e3));
 }
 
 template <typename L, bool RHO0, bool WALLS, bool MRT>

@@ -49,3 +49,22 @@ def test_the_decision_is_read_only():
     sim = _Handle((8, 8, 8))
     assert sim.lib.lbm_set_option(sim.h, _lib.OPT_STEPS_PER_PASS, 2.0) == _lib.LBM_EINVAL
     assert b"read only" in sim.lib.lbm_last_error(sim.h)
+
+
+# nx, ny, nz; whether LBM_OPT_STEP_PAIRS = 2 may run pairs: planes of 2^30 cells (32-bit byte offsets), edges of which
+# three do not fit an int, more tile rows (22 rows each, D3Q27 14) than a grid may have
+@pytest.mark.parametrize("shape,stencil,passes", [
+    ((32768, 32767, 1), 19, 2), ((32768, 32768, 1), 19, 1), ((32768, 33000, 1), 19, 1), ((40000, 30000, 1), 19, 1),
+    ((1 << 29, 1, 2), 19, 2), ((720000000, 1, 1), 19, 1), ((1, 720000000, 1), 19, 1),
+    ((2, 22 * 65535, 3), 19, 2), ((2, 22 * 65535 + 1, 3), 19, 1), ((2, 14 * 65535, 3), 27, 2),
+    ((2, 14 * 65535 + 1, 3), 27, 1), ((1, 1, 1), 19, 2)])
+def test_lattices_that_pairs_cannot_address_step_singly(shape, stencil, passes):
+    assert _Handle(shape, stencil, options=[(_lib.OPT_STEP_PAIRS, 2)]).option(_lib.OPT_STEPS_PER_PASS) == passes
+
+
+def test_offsets_of_the_largest_lattices_that_run_in_pairs():
+    """The kernel's coordinates and byte offsets, in Python: within int and unsigned for what the rule lets through."""
+    for nx, ny in ((32768, 32767), (1 << 29, 1), (1, 1 << 29), (1 << 15, (1 << 15) - 1)):
+        assert nx * ny < 1 << 30
+        assert (nx + 30) + 2 * nx < 1 << 31 and (ny + 30) + 2 * ny < 1 << 31  # (xr - 1 + i + 2 nx), yr alike
+        assert 4 * (nx * ny - 1) < 1 << 32                                    # ys[] + xs[]
