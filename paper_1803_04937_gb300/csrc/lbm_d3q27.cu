@@ -219,24 +219,12 @@ __global__ void __launch_bounds__(256) k27_ab1(const T *src, T *dst, Geo g,
 // A/B pull step for 16-bit storage, four cells per thread (nx % 4 == 0): the
 // same windowed quads as the D3Q19 four-cell step (each +-x shifted window
 // formed by funnel shifts from the aligned quad and its aligned neighbour),
-// 27 populations.  Bitwise the same results as k27_ab1.  FLAT as in k_aa_odd4
-// (256^3 FP16: 280 -> 268 us in rectangles).
-template <typename T, bool RHO0, bool WALLS, bool XONLY = false, bool FLAT = true>
-__global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g,
-                                                  Relax27<float> p, Box box)
+// 27 populations.  Bitwise the same results as k27_ab1.
+template <typename T, bool RHO0, bool WALLS>
+__device__ __forceinline__ void ab4_body27(const T *src, T *dst, const Site<WALLS> &s, const Geo &g,
+                                           const Relax27<float> &p)
 {
-    int xq, y, z;
-    if constexpr (FLAT) {
-        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-        if (i >= box.count) return;
-        if constexpr (WALLS && !XONLY) box.at_wall(i, xq, y, z);
-        else box.at(i, xq, y, z);
-    } else if (!box.at_block(xq, y, z)) {
-        return;
-    }
-    const int x0 = 4 * xq;
-    Site<WALLS> s(x0, y, z, 4, g);
-    drop_yz<XONLY>(s);
+    const int x0 = s.x;
     const int xprev = x0 == 0 ? g.nx - 4 : x0 - 4;
     const int xnext = x0 + 4 >= g.nx ? 0 : x0 + 4;
     const unsigned short *base = reinterpret_cast<const unsigned short *>(src);
@@ -296,7 +284,46 @@ __global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g,
 #pragma unroll
     for (int q = 0; q < Q27; ++q)
         *reinterpret_cast<uint2 *>(out + (long long)q * g.ncell + s.own + x0) = win[q];
-    if constexpr (WALLS && !XONLY) step_end(box);
+}
+
+// FLAT as in k27_ab1 (256^3 FP16: 280 -> 268 us in rectangles).
+template <typename T, bool RHO0, bool FLAT>
+__global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g, Relax27<float> p, Box box)
+{
+    int xq, y, z;
+    if constexpr (FLAT) {
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= box.count) return;
+        box.at(i, xq, y, z);
+    } else if (!box.at_block(xq, y, z)) {
+        return;
+    }
+    ab4_body27<T, RHO0>(src, dst, Site<false>(4 * xq, y, z, 4, g), g, p);
+}
+
+// With walls (WalledBox); XWALLS: walls on x too.
+template <typename T, bool RHO0, bool XWALLS, bool FLAT>
+__global__ void __launch_bounds__(128, 4) k27_ab4_walls(const T *src, T *dst, Geo g, Relax27<float> p, WalledBox box)
+{
+    int xq, y, z;
+    if (box.at_walls()) {
+        const unsigned i = box.wall_item();
+        if (i >= box.walls.count) return;
+        box.walls.at_wall(i, xq, y, z);
+        ab4_body27<T, RHO0>(src, dst, Site<true>(4 * xq, y, z, 4, g), g, p);
+        return;
+    }
+    if constexpr (FLAT) {
+        const unsigned i = box.inner_item();
+        if (i >= box.inner.count) return;
+        box.inner.at(i, xq, y, z);
+    } else {
+        box.inner_rectangle(xq, y, z);
+        if (xq >= (int)box.inner.per_row.d || y >= box.inner.y0 + (int)box.inner.rows.d) return;
+    }
+    Site<XWALLS> s(4 * xq, y, z, 4, g);
+    drop_yz(s);
+    ab4_body27<T, RHO0>(src, dst, s, g, p);
 }
 
 // The lattice for two FP32 steps per pass (k_pair).  16 rows leave 128 registers a
@@ -476,19 +503,23 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
         if constexpr (sizeof(T) == 2) {
             if (s.cells_x == 4 && g.nx % 4 == 0) {
                 // four cells per thread; with walls, the interior rows run the periodic
-                // kernel (or with walls on x the x-walls-only one) and the wall rows the
-                // walled one (split_rows): walled channel 512x256x256, FP16, 0.68 -> 1.0
-                // of the copy bandwidth
+                // code (or with walls on x the x-walls-only one) and the wall rows the
+                // walled one: walled channel 512x256x256, FP16, 0.68 -> 1.0 of the copy
+                // bandwidth
                 auto run = [&](auto rho0, auto walled) {
                     constexpr bool RH = decltype(rho0)::value, W = decltype(walled)::value;
-                    split_rows<W>(g, g.nx / 4, [&](int kind, const Box &box) {
-                        const int bx = kind == ROWS_WALLED ? 0 : box.block_x(QUAD_THREADS);
-                        auto k = kind == ROWS_WALLED ? q27::k27_ab4<T, RH, true>
-                                 : kind == ROWS_XWALLS
-                                     ? (bx ? q27::k27_ab4<T, RH, true, true, false> : q27::k27_ab4<T, RH, true, true>)
-                                     : (bx ? q27::k27_ab4<T, RH, false, false, false> : q27::k27_ab4<T, RH, false>);
-                        launch_step_box(k, box.beside, box, bx, QUAD_THREADS, stream, a, b, g, p);
-                    });
+                    if constexpr (W) {
+                        const WalledBox box(g.nx / 4, g.nx / 4, g, QUAD_THREADS, true);
+                        const bool flat = box.bx_log2 < 0;
+                        auto k = g.wall_x ? (flat ? q27::k27_ab4_walls<T, RH, true, true> : q27::k27_ab4_walls<T, RH, true, false>)
+                                          : (flat ? q27::k27_ab4_walls<T, RH, false, true> : q27::k27_ab4_walls<T, RH, false, false>);
+                        launch_step_walls(k, false, box, QUAD_THREADS, stream, a, b, g, p);
+                    } else {
+                        const Box box(g.nx / 4, 0, g.ny, 0, g.nz);
+                        const int bx = box.block_x(QUAD_THREADS);
+                        launch_step_box(bx ? q27::k27_ab4<T, RH, false> : q27::k27_ab4<T, RH, true>, false, box, bx, QUAD_THREADS,
+                                        stream, a, b, g, p);
+                    }
                 };
                 if (c.rho0_is_rho && walls) run(std::true_type{}, std::true_type{});
                 else if (c.rho0_is_rho) run(std::true_type{}, std::false_type{});

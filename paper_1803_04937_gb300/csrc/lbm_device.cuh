@@ -115,7 +115,7 @@ struct Box {
     Divider planes{1};      // ... and planes of a y face
     int y_last = 0, z_last = 0;
     int nz = 0;             // planes of the box
-    bool beside = false;    // runs beside the launch before it (see step_begin)
+    bool waits = true;      // step_begin waits for the launch before (false: it had ended before this one began)
 
     Box() = default;
     Box(int items_per_row, int y0_, int y1, int z0_, int planes_)
@@ -191,23 +191,61 @@ struct Box {
     }
 };
 
+// The rows of a lattice with walls in one launch: the first blocks take the rows at
+// walls normal to y or z (which cost more and so start first), the others the rows
+// between them, as one sequence of items or (bx_log2 >= 0) in blocks that are rectangles of
+// rows.  Every row is in exactly one block's part, and which part a block has is
+// uniform in it.
+struct WalledBox {
+    Box walls, inner;
+    unsigned wall_blocks;
+    int bx_log2;                  // -1: inner is one sequence
+    Divider blocks_x, blocks_y;   // rectangles along x and y
+
+    // rectangles: where the shape of the inner rows fills them (Box::block_x)
+    WalledBox(int items_per_row, int items_per_wall_row, const Geo &g, int threads, bool rectangles)
+        : walls(Box::wall_rows(items_per_wall_row, g))
+    {
+        const int ylo = g.wall_y ? 1 : 0, yhi = g.wall_y ? g.ny - 1 : g.ny;
+        const int zlo = g.wall_z ? 1 : 0, zhi = g.wall_z ? g.nz - 1 : g.nz;
+        const bool some = yhi > ylo && zhi > zlo;
+        inner = some ? Box(items_per_row, ylo, yhi, zlo, zhi - zlo) : Box(items_per_row, 0, 1, 0, 0);
+        wall_blocks = (walls.count + threads - 1) / threads;
+        const int bx = rectangles && some ? inner.block_x(threads) : 0;
+        bx_log2 = bx == 0 ? -1 : (bx == 128 ? 7 : (bx == 64 ? 6 : 5));
+        blocks_x = Divider(bx ? (int)((inner.per_row.d + bx - 1) / bx) : 1);
+        blocks_y = Divider(bx ? (int)((inner.rows.d + threads / bx - 1) / (threads / bx)) : 1);
+    }
+    unsigned blocks(int threads) const
+    {
+        return wall_blocks + (bx_log2 < 0 ? (inner.count + threads - 1) / threads : blocks_x.d * blocks_y.d * (unsigned)inner.nz);
+    }
+    __device__ __forceinline__ bool at_walls() const { return blockIdx.x < wall_blocks; }
+    // this thread's item in the sequence of its block's part
+    __device__ __forceinline__ unsigned wall_item() const { return blockIdx.x * blockDim.x + threadIdx.x; }
+    __device__ __forceinline__ unsigned inner_item() const { return (blockIdx.x - wall_blocks) * blockDim.x + threadIdx.x; }
+    // ... and its item, y and z in a rectangle; y may lie past the box, item past the row
+    __device__ __forceinline__ void inner_rectangle(int &item, int &y, int &z) const
+    {
+        int ix, iy;
+        z = inner.z0 + blocks_y.div(blocks_x.div((int)(blockIdx.x - wall_blocks), ix), iy);
+        item = (ix << bx_log2) + (int)(threadIdx.x & ((1u << bx_log2) - 1));
+        y = inner.y0 + iy * (int)(blockDim.x >> bx_log2) + (int)(threadIdx.x >> bx_log2);
+    }
+};
+
 // Launches of consecutive steps overlap their start with the end of the one
 // before (programmatic dependent launch): a step's blocks may be scheduled once
 // all blocks of the launch before have passed step_begin, that is once it needs
-// no more slots, and wait there for its completion.  A launch `beside` the one
-// before works on other rows of the same step: it reads what the step before
-// left, which the launch beside it has waited for, so it need not wait for that
-// one before its work but only before it ends, so that its own completion stands
-// for both.
+// no more slots, and wait there for its completion, which also makes visible what
+// it wrote.  Every launch that may start early waits for itself: another launch's
+// wait orders its blocks, but publishes no memory to them.
 __device__ __forceinline__ void step_begin(const Box &box)
 {
-    if (!box.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (box.waits) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-__device__ __forceinline__ void step_end(const Box &box)
-{
-    if (box.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-}
+__device__ __forceinline__ void step_begin(const WalledBox &box) { step_begin(box.inner); }
 
 // One lattice cell with its wrapped neighbour coordinates and the wall flags
 // of its six faces (true when the neighbour across that face is beyond a wall).

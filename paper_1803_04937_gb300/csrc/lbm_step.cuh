@@ -108,12 +108,12 @@ struct Site {
     }
 };
 
-// Rows that touch no y/z wall on a lattice with walls on x (XONLY kernels):
-// the y/z wall flags are constant false, so only the x-wall selects remain.
-template <bool XONLY, bool WALLS>
+// For rows that touch no y/z wall: the y/z wall flags are constant false, so
+// only the x-wall selects remain.
+template <bool WALLS>
 __device__ __forceinline__ void drop_yz(Site<WALLS> &s)
 {
-    if constexpr (XONLY) s.bym = s.byp = s.bzm = s.bzp = false;
+    s.bym = s.byp = s.bzm = s.bzp = false;
 }
 
 // An in-place step writes the locations it has read; left alone, the compiler
@@ -282,35 +282,62 @@ __global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(false)) k_aa_even1(Pla
 // AA odd step: read plane qbar at x - c_q, write plane q at x + c_q (through
 // a wall: read plane q / write plane qbar of the own cell).  Every location is
 // read and written by exactly one thread.
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
-__global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Planes<T> P, Geo g,
-                                                                         Relax<typename Storage<T>::R> p, Box box)
+template <typename T, bool RHO0, bool MRT, bool WALLS>
+__device__ __forceinline__ void aa_odd1_body(const Planes<T> &P, const Site<WALLS> &s,
+                                             const Relax<typename Storage<T>::R> &p)
 {
     using R = typename Storage<T>::R;
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= box.count) return;
-    int x, y, z;
-    if constexpr (WALLS && !XONLY) box.at_wall(i, x, y, z);
-    else box.at(i, x, y, z);
-    step_begin(box);
-    Site<WALLS> s(x, y, z, 1, g);
-    drop_yz<XONLY>(s);
     R f[Q];
     gather1<true>(P, s, f);
     collide_any<R, RHO0, MRT, one_rounding_v<T>>(f, p);
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int cx = CX(q);
-        const int xt = cx == 0 ? x : (cx > 0 ? s.xp : s.xm);
+        const int xt = cx == 0 ? s.x : (cx > 0 ? s.xp : s.xm);
         bool w = s.template wall_yz<1>(q);
         if (WALLS) {
             if (cx > 0) w |= s.bxp;
             if (cx < 0) w |= s.bxm;
         }
-        T *a = w ? P.p[OPP(q)] + s.own + x : P.p[q] + s.template row_along<1>(q) + xt;
+        T *a = w ? P.p[OPP(q)] + s.own + s.x : P.p[q] + s.template row_along<1>(q) + xt;
         Storage<T>::store(a, f[q]);
     }
-    if constexpr (WALLS && !XONLY) step_end(box);
+}
+
+template <typename T, bool RHO0, bool MRT = false>
+__global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1(Planes<T> P, Geo g,
+                                                                         Relax<typename Storage<T>::R> p, Box box)
+{
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= box.count) return;
+    int x, y, z;
+    box.at(i, x, y, z);
+    step_begin(box);
+    aa_odd1_body<T, RHO0, MRT>(P, Site<false>(x, y, z, 1, g), p);
+}
+
+// With walls (WalledBox); XWALLS: walls on x too.
+template <typename T, bool RHO0, bool MRT, bool XWALLS>
+__global__ void __launch_bounds__(256, aa1_blocks<T, MRT>(true)) k_aa_odd1_walls(Planes<T> P, Geo g,
+                                                                               Relax<typename Storage<T>::R> p,
+                                                                               WalledBox box)
+{
+    int x, y, z;
+    if (box.at_walls()) {
+        const unsigned i = box.wall_item();
+        if (i >= box.walls.count) return;
+        box.walls.at_wall(i, x, y, z);
+        step_begin(box);
+        aa_odd1_body<T, RHO0, MRT>(P, Site<true>(x, y, z, 1, g), p);
+    } else {
+        const unsigned i = box.inner_item();
+        if (i >= box.inner.count) return;
+        box.inner.at(i, x, y, z);
+        step_begin(box);
+        Site<XWALLS> s(x, y, z, 1, g);
+        drop_yz(s);
+        aa_odd1_body<T, RHO0, MRT>(P, s, p);
+    }
 }
 
 // ---------------------------------------------------------------- two cells per thread
@@ -322,9 +349,9 @@ struct PairAt {
     int x0, y, z;
     bool active, head, last;
 
-    __device__ __forceinline__ PairAt(const Box &box, bool wall_rows = false)
+    __device__ __forceinline__ explicit PairAt(const Box &box) : PairAt(box, blockIdx.x * blockDim.x + threadIdx.x) {}
+    __device__ __forceinline__ PairAt(const Box &box, unsigned i, bool wall_rows = false)
     {
-        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
         const int lane = threadIdx.x & 31;
         active = i < box.count;
         int xp;
@@ -428,14 +455,11 @@ __global__ void __launch_bounds__(256) k_aa_even2(Planes<T> P, Geo g, Relax<type
 // neighbouring segment is written by the edge lane as a scalar.  Through a
 // wall the value goes to plane qbar of the own cell.  Every location is
 // written by exactly one thread, as in the one-cell kernel.
-template <typename T, bool RHO0, bool WALLS, bool XONLY = false>
-__global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p, Box box)
+template <typename T, bool RHO0, bool WALLS>
+__device__ __forceinline__ void aa_odd2_body(const Planes<T> &P, const Site<WALLS> &s, const PairAt &at,
+                                             const Relax<typename Storage<T>::R> &p)
 {
     using R = typename Storage<T>::R;
-    const PairAt at(box, WALLS && !XONLY);
-    Site<WALLS> s(at.x0, at.y, at.z, 2, g);
-    drop_yz<XONLY>(s);
-    step_begin(box);
     const int x0 = at.x0;
     const bool active = at.active, head = at.head, last = at.last;
     R f0[Q], f1[Q];
@@ -483,7 +507,34 @@ __global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<ty
                 Storage<T>::store((WALLS && s.bxm) ? bnc + s.own + x0 : dst + trow + s.xm, f0[q]);
         }
     }
-    if constexpr (WALLS && !XONLY) step_end(box);
+}
+
+template <typename T, bool RHO0>
+__global__ void __launch_bounds__(256, 2) k_aa_odd2(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p, Box box)
+{
+    const PairAt at(box);
+    const Site<false> s(at.x0, at.y, at.z, 2, g);
+    step_begin(box);
+    aa_odd2_body<T, RHO0>(P, s, at, p);
+}
+
+// With walls, as k_aa_odd1_walls.
+template <typename T, bool RHO0, bool XWALLS>
+__global__ void __launch_bounds__(256, 2) k_aa_odd2_walls(Planes<T> P, Geo g, Relax<typename Storage<T>::R> p,
+                                                          WalledBox box)
+{
+    if (box.at_walls()) {
+        const PairAt at(box.walls, box.wall_item(), true);
+        const Site<true> s(at.x0, at.y, at.z, 2, g);
+        step_begin(box);
+        aa_odd2_body<T, RHO0>(P, s, at, p);
+    } else {
+        const PairAt at(box.inner, box.inner_item());
+        Site<XWALLS> s(at.x0, at.y, at.z, 2, g);
+        drop_yz(s);
+        step_begin(box);
+        aa_odd2_body<T, RHO0>(P, s, at, p);
+    }
 }
 
 // ---------------------------------------------------------------- four cells per thread (16-bit storage)
@@ -619,30 +670,41 @@ __device__ __forceinline__ void ab4_body(const Planes<T> &src, const Planes<T> &
         *reinterpret_cast<uint2 *>(reinterpret_cast<unsigned short *>(dst.p[q]) + s.own + s.x) = win[q];
 }
 
-// Resident blocks per SM for k_ab4.  The walled kernel runs only the rows at y and
-// z walls (split_rows); over a whole walled lattice FP16 was faster at four blocks
-// and BF16 at five (walled channel 512x256x256: FP16 82.9 -> 84.5 GLUPS at four,
-// BF16 79.9 -> 74.4).
-template <typename T, bool WALLS>
-constexpr int ab4_blocks = (WALLS && std::is_same_v<T, __half>) ? 4 : 5;
-
-// XONLY: rows that touch no y/z wall on a lattice with walls on x (a
-// cavity's interior rows): one body with the x-wall selects only, which cost
-// little (the end quads' shifted windows take the reflected own quad).
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false>
-__global__ void __launch_bounds__(128, ab4_blocks<T, WALLS && !XONLY>) k_ab4(Planes<T> src, Planes<T> dst, Geo g,
-                                                                              Relax<float> p, Box box)
+template <typename T, bool RHO0, bool MRT = false>
+__global__ void __launch_bounds__(128, 5) k_ab4(Planes<T> src, Planes<T> dst, Geo g, Relax<float> p, Box box)
 {
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= box.count) return;  // no lane needs another lane's data
     int xq, y, z;
-    if constexpr (WALLS && !XONLY) box.at_wall(i, xq, y, z);
-    else box.at(i, xq, y, z);
-    Site<WALLS> s(4 * xq, y, z, 4, g);
-    drop_yz<XONLY>(s);
+    box.at(i, xq, y, z);
+    const Site<false> s(4 * xq, y, z, 4, g);
     step_begin(box);
-    ab4_body<T, RHO0, WALLS, MRT>(src, dst, s, g, p);
-    if constexpr (WALLS && !XONLY) step_end(box);
+    ab4_body<T, RHO0, false, MRT>(src, dst, s, g, p);
+}
+
+// With walls (WalledBox); XWALLS: walls on x too, whose selects cost the rows
+// between the y and z walls little (the end quads' shifted windows take the
+// reflected own quad).
+template <typename T, bool RHO0, bool MRT, bool XWALLS>
+__global__ void __launch_bounds__(128, 5) k_ab4_walls(Planes<T> src, Planes<T> dst, Geo g, Relax<float> p, WalledBox box)
+{
+    int xq, y, z;
+    if (box.at_walls()) {
+        const unsigned i = box.wall_item();
+        if (i >= box.walls.count) return;
+        box.walls.at_wall(i, xq, y, z);
+        const Site<true> s(4 * xq, y, z, 4, g);
+        step_begin(box);
+        ab4_body<T, RHO0, true, MRT>(src, dst, s, g, p);
+    } else {
+        const unsigned i = box.inner_item();
+        if (i >= box.inner.count) return;
+        box.inner.at(i, xq, y, z);
+        Site<XWALLS> s(4 * xq, y, z, 4, g);
+        drop_yz(s);
+        step_begin(box);
+        ab4_body<T, RHO0, XWALLS, MRT>(src, dst, s, g, p);
+    }
 }
 
 // A/B pull step for 16-bit storage whose rows hold pairs but not quads of cells
@@ -735,7 +797,7 @@ __global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, 
 // quad goes to plane qbar of the own cells.  Each location is written by one
 // thread, and read (for a value that is used) only by that thread, as in the
 // one-cell kernel.
-// FORM: how the quads are walked.  ROWS_OF_BLOCKS: in blocks that are rectangles
+// FORM: how the quads are walked (SEQUENCE_CACHED on periodic lattices only).  ROWS_OF_BLOCKS: in blocks that are rectangles
 // of rows, whose rows a warp does not leave; the fastest from DRAM where rows fill
 // them (step of a pair, 256^3: FP16 208 us against 227, BF16 212 against 229).
 // SEQUENCE: as one sequence (192^3 FP16: 95 against 108 us, 160^3 60 against 74).
@@ -744,34 +806,64 @@ __global__ void __launch_bounds__(128, 5) k_aa_even4(Planes<T> P, Planes<T> Pw, 
 // spreads them among the collisions: that saves its spills, but leaves too few
 // loads in flight for DRAM (192^3 FP16: 99 us).
 enum OddForm { ROWS_OF_BLOCKS, SEQUENCE, SEQUENCE_CACHED };
-template <typename T, bool RHO0, bool WALLS, bool MRT = false, bool XONLY = false, OddForm FORM = SEQUENCE>
-__global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g, Relax<float> p, Box box)
+// With walls (WalledBox) the wall rows are stepped cell by cell, and the rows
+// between them keep the x-wall selects also without walls on x (the flags are then
+// false).  Both in one launch: a launch of its own for the wall rows after the other
+// costs a small lattice a second launch (closed box 32^3 FP16, step of a pair: 5.3
+// against 3.0 us; 96^3 15.6 against 11.7).  At four blocks per SM instead of five
+// nothing spills, and the branch is wanted by the rectangles only (256^3 with rho0 =
+// rho 262 us without it, 230 with; sequences of 192^3 FP16 93 us without, 105 with,
+// at five blocks 100).
+template <typename T, bool RHO0, bool WALLS, bool MRT = false, OddForm FORM = SEQUENCE>
+__global__ void __launch_bounds__(128, MRT || WALLS ? 4 : 5)
+    k_aa_odd4(Planes<T> P, Geo g, Relax<float> p, std::conditional_t<WALLS, WalledBox, Box> box)
 {
     const int lane = threadIdx.x & 31;
     constexpr bool SEQ = FORM != ROWS_OF_BLOCKS;
     int xq, y, z;
     bool active, end;  // end: the last quad there is for a warp that is not full
-    if constexpr (SEQ) {
+    if constexpr (WALLS) {
+        if (box.at_walls()) {
+            const unsigned i = box.wall_item();
+            if (i >= box.walls.count) return;
+            int x;
+            box.walls.at_wall(i, x, y, z);
+            aa_odd1_body<T, RHO0, MRT>(P, Site<true>(x, y, z, 1, g), p);
+            return;
+        }
+        if constexpr (SEQ) {
+            const unsigned i = box.inner_item();
+            active = i < box.inner.count;
+            end = i + 1 >= box.inner.count;
+            box.inner.at(active ? i : box.inner.count - 1u, xq, y, z);
+        } else {
+            box.inner_rectangle(xq, y, z);
+            if (y >= box.inner.y0 + (int)box.inner.rows.d) return;  // uniform across the warp
+            active = 4 * xq < g.nx;
+            xq = active ? xq : 0;
+            end = false;
+        }
+    } else if constexpr (SEQ) {
         const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
         active = i < box.count;
         end = i + 1 >= box.count;
-        if constexpr (WALLS && !XONLY) box.at_wall(active ? i : box.count - 1u, xq, y, z);
-        else box.at(active ? i : box.count - 1u, xq, y, z);
+        box.at(active ? i : box.count - 1u, xq, y, z);
     } else {
         const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-        y = (WALLS ? box.y0 : 0) + (int)(blockIdx.y * blockDim.y + threadIdx.y);
-        z = (WALLS ? box.z0 : 0) + (int)blockIdx.z;
-        if (y >= (WALLS ? box.y0 + (int)box.rows.d : g.ny)) return;  // uniform across the warp
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+        z = blockIdx.z;
+        if (y >= g.ny) return;  // uniform across the warp
         active = x0 < g.nx;
         xq = active ? x0 >> 2 : 0;
         end = false;
     }
     Site<WALLS> s(4 * xq, y, z, 4, g);
-    drop_yz<XONLY>(s);
+    drop_yz(s);
     // ends of the lanes' segment of a row (a warp of a sequence may hold several rows' ends)
     const bool head = lane == 0 || (SEQ && xq == 0);
     const bool last = lane == 31 || s.x + 4 >= g.nx || end;
-    if constexpr (FORM == SEQUENCE) step_begin(box);  // a branch that the loads stay behind; nothing to wait for
+    // a branch that the loads stay behind; nothing to wait for
+    if constexpr (FORM == (WALLS ? ROWS_OF_BLOCKS : SEQUENCE)) step_begin(box);
     uint2 quad[Q];
     load4w<true>(P, s, g, quad);
     if (active) collide4<T, RHO0, MRT>(quad, p);
@@ -828,49 +920,14 @@ __global__ void __launch_bounds__(128, MRT ? 4 : 5) k_aa_odd4(Planes<T> P, Geo g
                 *((WALLS && s.bxm) ? bnc + sw.own + sw.x : dst + trow + sw.xm) = (unsigned short)(quad[q].x & 0xffffu);
         }
     }
-    if constexpr (WALLS && !XONLY) step_end(box);
 }
 
 // ---------------------------------------------------------------- dispatch
 
-// Kinds of the launches of split_rows.
-enum { ROWS_PERIODIC = 0, ROWS_WALLED = 1, ROWS_XWALLS = 2 };
-
-// Calls launch(kind, box) for the launches of one step.  A periodic lattice is
-// one ROWS_PERIODIC launch over all rows.  With walls, the interior rows (no
-// link crosses a y or z wall) run the periodic kernel, or with walls on x the
-// kernel that has the x-wall selects only (ROWS_XWALLS), and the rows at y and z
-// walls the walled one (ROWS_WALLED) in one launch beside it; every row is in
-// exactly one launch, and no launch reads what the other writes.  All kernels
-// compute a cell with the same code, so the results are bitwise the same.  A
-// walled four-cell kernel over all rows carries both bodies and spills; keeping
-// it to the wall rows took the walled channel 512x256x256 from 84.3 to 89.1
-// GLUPS (FP16) and from 80.0 to 86.9 (BF16), and a cavity (walls on x, y and z)
-// 512x256x256 from 0.76 to 0.95 of the copy bandwidth (FP16 A/B).  One launch
-// for all wall rows that runs beside the interior one, instead of four after it:
-// closed box 32^3 FP16 A/B 14.2 -> 3.7 us a step, 128^3 41.3 -> 28.3.
-template <bool WALLS, typename F>
-static void split_rows(const Geo &g, int items_per_row, F &&launch)
-{
-    if (!WALLS) {
-        launch(ROWS_PERIODIC, Box(items_per_row, 0, g.ny, 0, g.nz));
-        return;
-    }
-    const int ylo = g.wall_y ? 1 : 0, yhi = g.wall_y ? g.ny - 1 : g.ny;
-    const int zlo = g.wall_z ? 1 : 0, zhi = g.wall_z ? g.nz - 1 : g.nz;
-    const bool interior = yhi > ylo && zhi > zlo;
-    if (interior) launch(g.wall_x ? ROWS_XWALLS : ROWS_PERIODIC, Box(items_per_row, ylo, yhi, zlo, zhi - zlo));
-    Box walls = Box::wall_rows(items_per_row, g);
-    walls.beside = interior;
-    if (walls.count) launch(ROWS_WALLED, walls);
-}
-
 static inline unsigned blocks_for(long long items, int threads) { return (unsigned)((items + threads - 1) / threads); }
 
 // Launches a step kernel; early: as a programmatic dependent of the stream's
-// last launch (step_begin).  Kernels with non-coherent loads are not launched
-// early, except beside a launch of the same step that was not, whose start
-// already followed the end of the step before.
+// last launch (step_begin).  Kernels with non-coherent loads are not launched early.
 template <typename... P, typename... A>
 static void launch_step_kernel(void (*kernel)(P...), bool early, dim3 grid, dim3 threads, cudaStream_t stream,
                                int shared_bytes, A &&...args)
@@ -891,9 +948,10 @@ static void launch_step_kernel(void (*kernel)(P...), bool early, dim3 grid, dim3
 // ... over a box, whose rows fill blocks of bx threads along x, or (bx = 0) as
 // one sequence of items; the box is the kernel's last argument.
 template <typename... P, typename... A>
-static void launch_step_box(void (*kernel)(P...), bool early, const Box &box, int bx, int threads, cudaStream_t stream,
+static void launch_step_box(void (*kernel)(P...), bool early, Box box, int bx, int threads, cudaStream_t stream,
                             A &&...args)
 {
+    box.waits = early;
     if (bx == 0) {
         launch_step_kernel(kernel, early, blocks_for(box.count, threads), threads, stream, 0, std::forward<A>(args)..., box);
         return;
@@ -901,6 +959,24 @@ static void launch_step_box(void (*kernel)(P...), bool early, const Box &box, in
     const unsigned ux = (unsigned)bx, uy = (unsigned)(threads / bx);
     launch_step_kernel(kernel, early, dim3((box.per_row.d + ux - 1) / ux, (box.rows.d + uy - 1) / uy, (unsigned)box.nz),
                        dim3(ux, uy), stream, 0, std::forward<A>(args)..., box);
+}
+
+// ... over a lattice with walls, whose interior rows (no link crosses a y or z wall)
+// run the periodic code, or with walls on x the code that has the x-wall selects
+// only, and whose rows at y and z walls run the walled one.  All of them compute a
+// cell with the same operations, so the results are bitwise the same.  Running the
+// walled code on the wall rows only took the walled channel 512x256x256 from 84.3 to
+// 89.1 GLUPS (FP16 A/B) and from 80.0 to 86.9 (BF16), and a cavity (walls on x, y and
+// z) 512x256x256 from 0.76 to 0.95 of the copy bandwidth.
+// One launch for all of them waits once for the step before; with the wall rows in a
+// launch of their own beside the other, closed boxes took 3.7 us a step at 32^3 (FP16
+// A/B; now 2.9) and 102 at 256x192x160 (BF16; now 97).
+template <typename... P, typename... A>
+static void launch_step_walls(void (*kernel)(P...), bool early, WalledBox box, int threads, cudaStream_t stream,
+                              A &&...args)
+{
+    box.inner.waits = early;
+    launch_step_kernel(kernel, early, box.blocks(threads), threads, stream, 0, std::forward<A>(args)..., box);
 }
 
 // The one-cell A/B step stays one launch over all rows: its walled kernel
@@ -919,19 +995,18 @@ static void launch_ab1(const Planes<T> &S, const Planes<T> &D, const Geo &g, con
 // over the SMs (32^3: 11.8 -> 19.4 us a step; the A/B step gains, 11.8 -> 10.8).
 template <typename T> constexpr bool aa1_early = sizeof(T) < 8;
 
-// The one-cell AA odd step, split into interior and wall rows like the
-// four-cell one (walled channel 512x256x256, FP32: odd step 0.72 of the copy
-// bandwidth as one walled launch).
+// The one-cell AA odd step, with the wall rows apart like the four-cell one
+// (walled channel 512x256x256, FP32: odd step 0.72 of the copy bandwidth with the
+// walled code on every row).
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_aa_odd1(const Planes<T> &P, const Geo &g, const Relax<typename Storage<T>::R> &p, int threads,
                            cudaStream_t stream)
 {
-    split_rows<WALLS>(g, g.nx, [&](int kind, const Box &box) {
-        auto k = kind == ROWS_WALLED   ? k_aa_odd1<T, RHO0, true, MRT>
-                 : kind == ROWS_XWALLS ? k_aa_odd1<T, RHO0, true, MRT, true>
-                                       : k_aa_odd1<T, RHO0, false, MRT>;
-        launch_step_box(k, aa1_early<T> || box.beside, box, 0, threads, stream, P, g, p);
-    });
+    if constexpr (WALLS)
+        launch_step_walls(g.wall_x ? k_aa_odd1_walls<T, RHO0, MRT, true> : k_aa_odd1_walls<T, RHO0, MRT, false>, aa1_early<T>,
+                          WalledBox(g.nx, g.nx, g, threads, false), threads, stream, P, g, p);
+    else
+        launch_step_box(k_aa_odd1<T, RHO0, MRT>, aa1_early<T>, Box(g.nx, 0, g.ny, 0, g.nz), 0, threads, stream, P, g, p);
 }
 
 constexpr int QUAD_THREADS = 128;  // threads per block of the four-cell kernels
@@ -939,39 +1014,36 @@ constexpr int QUAD_THREADS = 128;  // threads per block of the four-cell kernels
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_ab4(const Planes<T> &S, const Planes<T> &D, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, g.nx / 4, [&](int kind, const Box &box) {
-        auto k = kind == ROWS_WALLED   ? k_ab4<T, RHO0, true, MRT>
-                 : kind == ROWS_XWALLS ? k_ab4<T, RHO0, true, MRT, true>
-                                       : k_ab4<T, RHO0, false, MRT>;
-        launch_step_box(k, true, box, 0, QUAD_THREADS, stream, S, D, g, p);
-    });
+    if constexpr (WALLS)
+        launch_step_walls(g.wall_x ? k_ab4_walls<T, RHO0, MRT, true> : k_ab4_walls<T, RHO0, MRT, false>, true,
+                          WalledBox(g.nx / 4, g.nx / 4, g, QUAD_THREADS, false), QUAD_THREADS, stream, S, D, g, p);
+    else
+        launch_step_box(k_ab4<T, RHO0, MRT>, true, Box(g.nx / 4, 0, g.ny, 0, g.nz), 0, QUAD_THREADS, stream, S, D, g, p);
 }
 
-// The four-cell AA odd step, split into interior and wall rows as the A/B
-// step is (split_rows): the walled kernel spills and runs the walled channel
-// 512x256x256's odd step at 0.55 of the copy bandwidth (FP16 and BF16) as one
-// launch.  Each location is read and written by one cell's thread only, so
-// the launches may run in any order.
+// The four-cell AA odd step, with the wall rows apart: four cells a thread with the
+// selects of all walls spill, and ran the walled channel 512x256x256's odd step at
+// 0.55 of the copy bandwidth (FP16 and BF16).  Each location is read and written by one cell's
+// thread only, so the blocks may run in any order.
 template <typename T, bool RHO0, bool WALLS, bool MRT>
 static void launch_aa_odd4(const Planes<T> &P, const Geo &g, const Relax<float> &p, cudaStream_t stream)
 {
-    split_rows<WALLS>(g, g.nx / 4, [&](int kind, const Box &box) {
+    if constexpr (WALLS) {
+        const WalledBox box(g.nx / 4, g.nx, g, QUAD_THREADS, true);
+        launch_step_walls(box.bx_log2 < 0 ? k_aa_odd4<T, RHO0, true, MRT> : k_aa_odd4<T, RHO0, true, MRT, ROWS_OF_BLOCKS>, false,
+                          box, QUAD_THREADS, stream, P, g, p);
+    } else {
+        const Box box(g.nx / 4, 0, g.ny, 0, g.nz);
         // the form for grids that stay in L2 (129 MB, with the next step's share)
         // serves periodic lattices only (128^3 with walls: 33.4 us, 29.1 in blocks)
-        const bool cached = !WALLS && g.ncell * Q * (long long)sizeof(T) < (100LL << 20);
-        const int bx = kind == ROWS_WALLED || cached ? 0 : box.block_x(QUAD_THREADS);
+        const bool cached = g.ncell * Q * (long long)sizeof(T) < (100LL << 20);
+        const int bx = cached ? 0 : box.block_x(QUAD_THREADS);
         // BF16 takes that form for every sequence (192^3: 101 against 103 us)
         constexpr OddForm seq = std::is_same_v<T, __nv_bfloat16> ? SEQUENCE_CACHED : SEQUENCE;
-        // the interior rows of a walled lattice take the x-walls-only kernel also
-        // without x walls (its x flags are then false): it compiles to a faster
-        // step than the periodic kernel with a row range (walled channel, FP16 AA
-        // pair 0.81 -> 0.85, BF16 0.80 -> 0.82)
-        auto k = kind == ROWS_WALLED ? k_aa_odd4<T, RHO0, true, MRT>
-                 : WALLS  ? (bx ? k_aa_odd4<T, RHO0, true, MRT, true, ROWS_OF_BLOCKS> : k_aa_odd4<T, RHO0, true, MRT, true>)
-                 : cached ? k_aa_odd4<T, RHO0, false, MRT, false, SEQUENCE_CACHED>
-                          : (bx ? k_aa_odd4<T, RHO0, false, MRT, false, ROWS_OF_BLOCKS> : k_aa_odd4<T, RHO0, false, MRT, false, seq>);
-        launch_step_box(k, box.beside, box, bx, QUAD_THREADS, stream, P, g, p);
-    });
+        auto k = cached ? k_aa_odd4<T, RHO0, false, MRT, SEQUENCE_CACHED>
+                        : (bx ? k_aa_odd4<T, RHO0, false, MRT, ROWS_OF_BLOCKS> : k_aa_odd4<T, RHO0, false, MRT, seq>);
+        launch_step_box(k, false, box, bx, QUAD_THREADS, stream, P, g, p);
+    }
 }
 
 // One-cell step of either pattern.
@@ -1030,13 +1102,13 @@ static cudaError_t step_t(int kind, void *src, void *dst, const Geo &g, const Co
         }
         else if (kind == 1)
             launch_step_box(k_aa_even2<T, RHO0>, true, box, 0, threads, stream, D, g, p);
-        else
-            split_rows<WALLS>(g, g.nx / 2, [&](int rows, const Box &part) {
-                auto k = rows == ROWS_WALLED   ? k_aa_odd2<T, RHO0, true>
-                         : rows == ROWS_XWALLS ? k_aa_odd2<T, RHO0, true, true>
-                                               : k_aa_odd2<T, RHO0, false>;
-                launch_step_box(k, true, part, 0, threads, stream, D, g, p);
-            });
+        else {
+            if constexpr (WALLS)
+                launch_step_walls(g.wall_x ? k_aa_odd2_walls<T, RHO0, true> : k_aa_odd2_walls<T, RHO0, false>, true,
+                                  WalledBox(g.nx / 2, g.nx / 2, g, threads, false), threads, stream, D, g, p);
+            else
+                launch_step_box(k_aa_odd2<T, RHO0>, true, box, 0, threads, stream, D, g, p);
+        }
         return cudaGetLastError();
     }
     if (cb.mrt)
