@@ -249,7 +249,9 @@ int lbm_moments(lbm_handle h, void *rho, void *u, int dtype);
 
 /*
  * FP64 reductions of the current state into host out[LBM_RED_COUNT] (slots
- * LBM_RED_*), deterministic for a given lattice size.  Needs a bound scratch
+ * LBM_RED_*), deterministic for a given lattice size.  Terms of FP32 arithmetic
+ * are summed to at least FP64's 53 bits (in threes of FP32 numbers, about 70 bits, for
+ * up to 64 cells of a thread, then in FP64); FP64 storage is summed in FP64.  Needs a bound scratch
  * buffer.  Synchronises the bound stream.  Returns LBM_ENONFINITE (with out
  * filled) if any population is NaN or Inf.
  */
@@ -259,11 +261,11 @@ int lbm_reduce(lbm_handle h, double *out);
  * Enstrophy of the current state into host *out: 1/2 <|curl u|^2>, the mean
  * over all cells, with u from Eq. 17 and second-order central differences
  * (u(x + e_a) - u(x - e_a)) / 2.  Periodic axes wrap; across a half-way
- * bounce-back wall the ghost velocity is -u of the own cell.  FP64
- * accumulation, deterministic for a given lattice size.  Needs a bound scratch
- * buffer; synchronises the bound stream.  D3Q19 only.  Off the per-step path:
- * each cell reads its six axis neighbours' populations.  Returns
- * LBM_ENONFINITE if the result is not finite.
+ * bounce-back wall the ghost velocity is -u of the own cell.  Summed as lbm_reduce
+ * sums, deterministic for a given lattice size.  Needs a bound scratch buffer;
+ * synchronises the bound stream.  D3Q19 only.  Off the per-step path: reads every
+ * population once, and those of the cells around each tile of 30 x 14 columns again.
+ * Returns LBM_ENONFINITE if the result is not finite.
  */
 int lbm_enstrophy(lbm_handle h, double *out);
 

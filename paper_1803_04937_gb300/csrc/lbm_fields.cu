@@ -152,27 +152,38 @@ __global__ void k_set(T *grid, const T *__restrict__ src, Geo g, Box box)
 // ---------------------------------------------------------------- reductions
 
 constexpr int RED_THREADS = 256;
-constexpr int RED_SMS = 152, RED_BLOCKS = RED_SMS * 4;  // all resident at once
+// All resident at once.  Three blocks per SM, whose 85 registers a thread the sums need:
+// lbm_reduce of 192^3 FP16 (whole call) 151 us, four blocks 160 (spills), five 169.
+constexpr int RED_SMS = 152, RED_PER_SM = 3, RED_BLOCKS = RED_SMS * RED_PER_SM;
 int reduce_blocks() { return RED_BLOCKS; }
 
 // A running sum.  This GPU adds about 64 FP32 numbers in the time of one FP64
-// number, so cells of FP32 arithmetic are summed in double-float (TwoSum; exact
-// products by fma), which keeps more bits of such terms than they have, and the
-// few cells' sum is added to an FP64 total before its own rounding matters.
+// number, so cells of FP32 arithmetic are summed exactly in FP32: as an unevaluated
+// sum hi + lo + rest, whose two leading parts take every rounding error (TwoSum;
+// exact products by fma) and whose last one, of the order of 2^-48 of the sum, is
+// rounded.  That keeps about 70 bits of a few cells, whose sum is then added to an
+// FP64 total: fewer FP64 roundings than adding every cell to it.  (hi + lo alone, 48
+// bits, fell short of FP64 sums.)
 template <typename R> struct Sum;
 template <> struct Sum<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v) { two_sum_acc(hi, lo, v); }
+    float hi = 0.f, lo = 0.f, rest = 0.f;
+    __device__ __forceinline__ void add_low(float v) { two_sum_acc(lo, rest, v); }
+    __device__ __forceinline__ void add(float v)
+    {
+        float e = 0.f;
+        two_sum_acc(hi, e, v);
+        add_low(e);
+    }
     __device__ __forceinline__ void add_product(float a, float b)
     {
         const float p = __fmul_rn(a, b);
-        two_sum_acc(hi, lo, p);
-        lo += fmaf(a, b, -p);
+        add(p);
+        add_low(fmaf(a, b, -p));
     }
     __device__ __forceinline__ void flush(double &total)
     {
-        total += (double)hi + (double)lo;
-        hi = lo = 0.f;
+        total += (double)hi + ((double)lo + (double)rest);
+        hi = lo = rest = 0.f;
     }
 };
 template <> struct Sum<double> {
@@ -185,7 +196,7 @@ template <> struct Sum<double> {
         v = 0.0;
     }
 };
-constexpr int SUM_CELLS = 16;  // cells between two flushes
+constexpr int SUM_CELLS = 64;  // cells between two flushes (with 16, lbm_reduce takes 6 % longer)
 
 // Whether products of FP32 numbers whose largest square is about v can be split
 // into value and rounding error in FP32: not where they come near its range's
@@ -207,10 +218,10 @@ __device__ __forceinline__ double warp_sum_or_max(double v, bool largest)
 // block of a fixed grid, in a fixed order (deterministic for a lattice size).
 // The kernel was bound by FP64 work, about 45 operations a cell (a square root
 // among them) and a 64-bit division; with the sums above, the root taken of the
-// thread's largest |u|^2 only and the row found by a multiplication it is bound
-// by its loads.
+// thread's largest |u|^2 only and the row found by a multiplication a call takes 151
+// instead of 397 us at 192^3 FP16, whose bytes take 40 at the copy bandwidth.
 template <typename T, int L, bool WALLS>
-__global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
+__global__ void __launch_bounds__(RED_THREADS, RED_PER_SM)
     k_reduce(Planes<T> P, double *partial, Geo g, Coll<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
@@ -218,7 +229,14 @@ __global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
     double acc[5] = {0, 0, 0, 0, 0}, uumax = 0.0;  // drho, |u|^2, rho0 u; largest |u|^2
     Sum<R> sum[5];
     R near_max = R(-1);  // |u|^2 below this cannot be the largest
-    int bad = 0, n = 0;
+    int bad = 0, n = 0, summed = 0;  // summed: cells in sum[] since the last flush
+    auto flush = [&] {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) sum[2 + i].add_product(R(-summed), p.half_a[i]);  // rho0 u = j + a/2
+#pragma unroll
+        for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
+        summed = 0;
+    };
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncell;
          cell += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
@@ -236,6 +254,7 @@ __global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
         const R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         bad += !finite;
         if (finite && fits_products(uu) && isfinite(drho)) {
+            ++summed;
             sum[0].add(drho);
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
@@ -250,7 +269,7 @@ __global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 acc[1] += (double)u[i] * (double)u[i];
-                acc[2 + i] += (double)rho0 * (double)u[i];
+                acc[2 + i] += (double)rho0 * (double)u[i] - (double)p.half_a[i];
             }
         }
         if (!(uu < near_max)) {
@@ -258,16 +277,10 @@ __global__ void __launch_bounds__(RED_THREADS, RED_BLOCKS / RED_SMS)
             uumax = fmax(uumax, v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
             near_max = R(uumax) * R(0.999999);
         }
-        if (++n % SUM_CELLS == 0) {
-#pragma unroll
-            for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
-        }
+        if (++n % SUM_CELLS == 0) flush();
     }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
+    flush();
     acc[1] *= 0.5;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) acc[2 + i] -= n * (double)p.half_a[i];  // rho0 u = j + a/2
     // one warp per result sums the block's threads (a shuffle tree of every warp
     // for every result would cost four times the FP64 additions)
     const double slot[7] = {acc[0], acc[1], acc[2], acc[3], acc[4], sqrt(uumax), (double)bad};
@@ -313,7 +326,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *part
 // registers and shares the middle one through shared memory.  (Gathering all
 // six neighbours' populations instead took 133 loads a cell and FP64
 // differences: 192^3 FP16 1.2 ms.)  Differences of FP32 velocities are taken
-// exactly in double-float, FP64 storage uses FP64.  Deterministic: fixed grid,
+// and squared to about 70 bits (Sum): a call at 192^3 takes 238 us (657 before the tiles;
+// 190 with 48-bit terms, which fall short of FP64); FP64 storage uses FP64.  Deterministic: fixed grid,
 // fixed tiles, fixed per-thread order, fixed trees.
 constexpr int ENS_LANES = 32, ENS_ROWS = 16, ENS_THREADS = ENS_LANES * ENS_ROWS;
 constexpr int ENS_X = ENS_LANES - 2, ENS_Y = ENS_ROWS - 2;
@@ -347,11 +361,23 @@ __device__ __forceinline__ DF exact_diff(float a, float b)
 // (a1 - a0) - (b1 - b0), twice a component of the curl, squared and added to s or total
 __device__ __forceinline__ void add_square_of_curl(Sum<float> &s, double &total, float a1, float a0, float b1, float b0)
 {
-    const DF w = df_add(exact_diff(a1, a0), exact_diff(b0, b1));
-    if (fits_products(w.hi * w.hi)) {
-        s.add_product(w.hi, w.hi);
-        s.lo = fmaf(2.f * w.hi, w.lo, s.lo);
-    } else if (w.hi != 0.f) {
+    const DF a = exact_diff(a1, a0), b = exact_diff(b0, b1);
+    // w = hi + lo + rest, the leading parts exact
+    float hi = a.hi, e = 0.f, lo = a.lo, rest = 0.f;
+    two_sum_acc(hi, e, b.hi);
+    two_sum_acc(lo, rest, b.lo);
+    two_sum_acc(lo, rest, e);
+    // (hi is a multiple of half the last bit of a.hi or b.hi, and so of lo's last bit:
+    // then hi + lo without TwoSum's second half is exact also where |lo| > |hi|)
+    const float w = hi + lo;
+    lo -= w - hi;
+    if (fits_products(w * w)) {
+        // w^2 + 2 w lo + (2 w rest + lo^2), by size of the parts
+        const float twice = 2.f * w, p = __fmul_rn(twice, lo);
+        s.add_product(w, w);
+        s.add_low(p);
+        s.rest += fmaf(twice, rest, fmaf(lo, lo, fmaf(twice, lo, -p)));
+    } else if (w != 0.f) {
         const double v = ((double)a1 - (double)a0) - ((double)b1 - (double)b0);
         total += v * v;
     }
