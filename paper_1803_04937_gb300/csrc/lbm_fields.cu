@@ -180,9 +180,10 @@ template <> struct Sum<float> {
         add(p);
         add_low(fmaf(a, b, -p));
     }
-    __device__ __forceinline__ void flush(double &total)
+    // adds the sum less `minus` to the total
+    __device__ __forceinline__ void flush(double &total, double minus = 0.0)
     {
-        total += (double)hi + ((double)lo + (double)rest);
+        total += ((double)hi - minus) + ((double)lo + (double)rest);
         hi = lo = rest = 0.f;
     }
 };
@@ -190,9 +191,9 @@ template <> struct Sum<double> {
     double v = 0.0;
     __device__ __forceinline__ void add(double x) { v += x; }
     __device__ __forceinline__ void add_product(double a, double b) { v = fma(a, b, v); }
-    __device__ __forceinline__ void flush(double &total)
+    __device__ __forceinline__ void flush(double &total, double minus = 0.0)
     {
-        total += v;
+        total += v - minus;
         v = 0.0;
     }
 };
@@ -203,6 +204,16 @@ constexpr int SUM_CELLS = 64;  // cells between two flushes (with 16, lbm_reduce
 // ends (nor for NaN); those few cells are summed in FP64 at once.
 __device__ __forceinline__ bool fits_products(float v) { return v > 1e-20f && v < 1e30f; }
 __device__ __forceinline__ bool fits_products(double v) { return isfinite(v); }
+// ... and whether a group's sum of such values v stays far from overflow
+__device__ __forceinline__ bool fits_sum(float v) { return fabsf(v) < 1e15f; }
+__device__ __forceinline__ bool fits_sum(double v) { return isfinite(v); }
+// ... and whether one product's rounding error is a normal number (or zero)
+__device__ __forceinline__ bool exact_product(float a, float b)
+{
+    const float p = fabsf(a * b);
+    return p > 1e-30f || a == 0.f || b == 0.f;
+}
+__device__ __forceinline__ bool exact_product(double, double) { return true; }
 
 __device__ __forceinline__ double warp_sum_or_max(double v, bool largest)
 {
@@ -231,10 +242,10 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM)
     R near_max = R(-1);  // |u|^2 below this cannot be the largest
     int bad = 0, n = 0, summed = 0;  // summed: cells in sum[] since the last flush
     auto flush = [&] {
+        sum[0].flush(acc[0]);
+        sum[1].flush(acc[1]);
 #pragma unroll
-        for (int i = 0; i < 3; ++i) sum[2 + i].add_product(R(-summed), p.half_a[i]);  // rho0 u = j + a/2
-#pragma unroll
-        for (int k = 0; k < 5; ++k) sum[k].flush(acc[k]);
+        for (int i = 0; i < 3; ++i) sum[2 + i].flush(acc[2 + i], summed * (double)p.half_a[i]);  // rho0 u = j + a/2
         summed = 0;
     };
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < g.ncell;
@@ -253,7 +264,12 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM)
         }
         const R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
         bad += !finite;
-        if (finite && fits_products(uu) && isfinite(drho)) {
+        bool fits = finite && fits_products(uu) && fits_sum(drho);
+        if (p.rho0_is_rho) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) fits &= exact_product(rho0, u[i]);
+        }
+        if (fits) {
             ++summed;
             sum[0].add(drho);
 #pragma unroll

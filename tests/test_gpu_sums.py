@@ -135,3 +135,31 @@ def test_enstrophy_is_no_less_precise_than_an_fp64_sum(shape, walls, precision):
         # (a difference of FP64 velocities may cancel: for that storage relative to the velocities)
         scale = float(want) if precision != "f64" else float(want) + float((u ** 2).max())
         assert abs(Fraction(sim.enstrophy()) - want) <= (7 + 6) * EPS * scale
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_sums_of_huge_finite_cells(precision):
+    """A diverging state whose cells are finite: the sum of two densities leaves FP32's range, not FP64's."""
+    sim = _sim((128, 64, 64), precision)  # more cells than threads
+    f = torch.zeros((19, 64, 64, 128), dtype=sim.storage_dtype, device="cuda")
+    f[0] = 3e38
+    f[1] = 0.01  # an ordinary velocity
+    sim.set_pdfs(f)
+    r = sim.reduce()
+    value = float(f[0, 0, 0, 0].double())
+    assert r["nonfinite"] == 0
+    assert abs(r["mass"] - value * sim.ncell) <= 48 * EPS * value * sim.ncell
+
+
+@pytest.mark.parametrize("force", [(0.0, 0.0, 0.0), (1e-3, 3e-33, 0.0)])
+def test_momentum_of_a_tiny_component_beside_an_ordinary_one(force):
+    """rho u_y of about 1e-33: the rounding error of that product is no normal FP32 number."""
+    sim = _sim((2, 2, 1), "f32", rho0=True, force=force)
+    for seed in range(24):
+        rng = np.random.default_rng(seed)
+        f = np.zeros((19,) + sim.shape)
+        f[0] = 0.05 * rng.standard_normal(sim.shape)
+        f[1] = 0.01 * rng.standard_normal(sim.shape)
+        f[3] = 1e-33 * rng.standard_normal(sim.shape)
+        sim.set_pdfs(torch.from_numpy(f).float())
+        _check(sim, True, force, levels=4)
