@@ -215,6 +215,12 @@ __device__ __forceinline__ bool exact_product(float a, float b)
 }
 __device__ __forceinline__ bool exact_product(double, double) { return true; }
 
+// A bound below v, the largest |u|^2 so far, so far off that the squares of a cell below
+// it cannot be larger in exact arithmetic; where squares of R lose bits near the end of its
+// range, none.
+__device__ __forceinline__ float near_square(float v) { return fits_products(v) ? v * 0.999999f : -1.f; }
+__device__ __forceinline__ double near_square(double v) { return v > 1e-280 ? v * 0.999999 : -1.0; }
+
 __device__ __forceinline__ double warp_sum_or_max(double v, bool largest)
 {
 #pragma unroll
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(RED_THREADS, RED_PER_SM)
         if (!(uu < near_max)) {
             const double v[3] = {(double)u[0], (double)u[1], (double)u[2]};
             uumax = fmax(uumax, v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-            near_max = R(uumax) * R(0.999999);
+            near_max = near_square(R(uumax));
         }
         if (++n % SUM_CELLS == 0) flush();
     }

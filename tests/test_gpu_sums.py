@@ -163,3 +163,16 @@ def test_momentum_of_a_tiny_component_beside_an_ordinary_one(force):
         f[3] = 1e-33 * rng.standard_normal(sim.shape)
         sim.set_pdfs(torch.from_numpy(f).float())
         _check(sim, True, force, levels=4)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-19, 1e-23])
+def test_umax_of_tiny_velocities(scale):
+    """Squares of FP32 velocities near or below FP32's smallest number: the largest |u| is still the largest.  The two
+    cells are one thread's (three blocks of 256 threads on each of 152 SMs)."""
+    threads = 152 * 3 * 256
+    sim = _sim((threads // 64, 64, 2), "f32")
+    f = torch.zeros((19, 2, 64, threads // 64), dtype=torch.float32, device="cuda")
+    f[1, 0, 0, 0] = 3.0 * scale                                # |u| = 3 scale
+    f[1, 1, 0, 0] = f[3, 1, 0, 0] = f[5, 1, 0, 0] = 2.5 * scale  # |u| = 4.33 scale
+    sim.set_pdfs(f)
+    assert sim.reduce()["umax"] == pytest.approx(2.5 * scale * 3 ** 0.5, rel=1e-6, abs=0.0)
