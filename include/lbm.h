@@ -107,7 +107,8 @@ typedef struct lbm_ctx *lbm_handle;
 #define LBM_OPT_BLOCK_X   13  /* step kernel threads per block along x (tuning) */
 #define LBM_OPT_BLOCK_Y   14  /* ... along y; bx * by <= 256 and a multiple of 32.  The one-cell
                                  kernels walk the lattice as one sequence of cells in blocks of
-                                 bx * by (if neither was set: of a size the library chooses) */
+                                 bx * by.  The values that a new handle reports stand for a size
+                                 the library chooses, also when they are set again */
 #define LBM_OPT_CELLS_X   15  /* cells per thread along x in the step kernel: 1; 2 (paired
                                  accesses; nx even, bx a multiple of 32); or 4 (16-bit storage,
                                  A/B and AA, nx a multiple of 4; otherwise
@@ -125,7 +126,7 @@ typedef struct lbm_ctx *lbm_handle;
 #define LBM_OPT_STEP_PAIRS 20 /* 1 (default): lbm_step computes two time steps per pass over the
                                  grids (the state between them stays on the chip) where that is
                                  faster: A/B pattern, FP32 storage, LBM_OPT_CELLS_X = 1, no
-                                 LBM_OPT_BLOCK_* set, larger lattices; 0: never; 2: for every
+                                 other LBM_OPT_BLOCK_* set, larger lattices; 0: never; 2: for every
                                  size of such a lattice but those the kernel cannot address (nx ny
                                  from 2^30 on, nx or ny above 2^29, or ny above about 900,000),
                                  which step singly.  The same populations either way, in the

@@ -24,7 +24,7 @@ struct lbm_ctx {
     int rho0_mode = 0;
     int pattern = LBM_PATTERN_AB;
     int bx = 128, by = 2;
-    bool block_set = false;  // the caller chose bx or by
+    bool block_set = false;  // the caller chose another block than a new handle reports
     int cells_x = 1;
     int pairs = 1;                                 // two steps per pass: 0 never, 1 where it pays, 2 always
     int graphs = 1;                                // replay GRAPH_STEPS-step CUDA graphs in lbm_step
@@ -93,6 +93,14 @@ int block_threads(const lbm_ctx *h)
 {
     if (h->precision == LBM_F64) return 32;
     return h->stencil == LBM_D3Q27 && ncell(h) >= (1 << 20) ? 256 : 128;
+}
+
+// The block that a new handle reports (LBM_OPT_BLOCK_X, _Y): it stands for the
+// library's own choice (block_threads).
+void default_block(int nx, int &bx, int &by)
+{
+    bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
+    by = 256 / bx;
 }
 
 double omega_minus(const lbm_ctx *h)
@@ -362,10 +370,7 @@ int lbm_create(int nx, int ny, int nz, int stencil, int equilibrium, int collisi
     h->collision = collision;
     h->tau = tau;
     h->precision = precision;
-    if (nx < 128) {
-        h->bx = nx <= 32 ? 32 : (nx <= 64 ? 64 : 128);
-        h->by = 256 / h->bx;
-    }
+    default_block(nx, h->bx, h->by);
     // 16-bit storage needs wide accesses shared by several cells to approach
     // the bandwidth roofline: four cells per thread (A/B and AA)
     h->cells_x = (precision == LBM_F16S || precision == LBM_BF16S) ? 4 : 1;
@@ -460,7 +465,8 @@ int lbm_set_option(lbm_handle h, int key, double v)
             return fail(h, LBM_EINVAL, "block must satisfy bx * by <= 256 and a multiple of 32");
         h->bx = bx;
         h->by = by;
-        h->block_set = true;
+        default_block(h->nx, bx, by);
+        h->block_set = h->bx != bx || h->by != by;
         return LBM_OK;
     }
     }

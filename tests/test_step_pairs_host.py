@@ -68,3 +68,17 @@ def test_offsets_of_the_largest_lattices_that_run_in_pairs():
         assert nx * ny < 1 << 30
         assert (nx + 30) + 2 * nx < 1 << 31 and (ny + 30) + 2 * ny < 1 << 31  # (xr - 1 + i + 2 nx), yr alike
         assert 4 * (nx * ny - 1) < 1 << 32                                    # ys[] + xs[]
+
+
+@pytest.mark.parametrize("nx", [24, 48, 100, 256])
+def test_setting_the_reported_block_again_keeps_the_librarys_choice(nx):
+    sim = _Handle((nx, 512, 512))
+    before = sim.option(_lib.OPT_STEPS_PER_PASS)
+    bx, by = sim.option(_lib.OPT_BLOCK_X), sim.option(_lib.OPT_BLOCK_Y)
+    for key, value in ((_lib.OPT_BLOCK_X, bx), (_lib.OPT_BLOCK_Y, by)):
+        assert sim.lib.lbm_set_option(sim.h, key, value) == 0
+        assert sim.option(_lib.OPT_STEPS_PER_PASS) == before
+    assert sim.lib.lbm_set_option(sim.h, _lib.OPT_BLOCK_Y, 1.0) == 0  # another block: one step per pass
+    assert sim.option(_lib.OPT_STEPS_PER_PASS) == 1
+    assert sim.lib.lbm_set_option(sim.h, _lib.OPT_BLOCK_Y, by) == 0
+    assert sim.option(_lib.OPT_STEPS_PER_PASS) == before
