@@ -176,10 +176,12 @@ __device__ __forceinline__ void collide27(R g[Q27], const Relax27<R> &p)
 }
 
 // A/B pull step, one cell per thread.  FLAT: the cells as one sequence, or in
-// blocks that are rectangles of rows, which is faster with walls where rows fill
-// them (256^3 FP32: 538 -> 524 us) and slower without.
+// blocks that are rectangles of rows, which is faster with walls where rows are
+// multiples of 128 cells (256^3 FP32: 549 -> 536 us) and slower elsewhere (513x100x100:
+// 170 -> 205).  Four blocks per SM, also with rho0 = rho (left alone, 73 registers and
+// three blocks: 259x307x95 with walls 325 us, 260 now).
 template <typename T, bool RHO0, bool WALLS, bool FLAT = true>
-__global__ void __launch_bounds__(256) k27_ab1(const T *src, T *dst, Geo g,
+__global__ void __launch_bounds__(256, sizeof(typename Storage<T>::R) == 4 ? 4 : 1) k27_ab1(const T *src, T *dst, Geo g,
                                                Relax27<typename Storage<T>::R> p, Box box)
 {
     using R = typename Storage<T>::R;
@@ -301,8 +303,9 @@ __global__ void __launch_bounds__(128, 4) k27_ab4(const T *src, T *dst, Geo g, R
     ab4_body27<T, RHO0>(src, dst, Site<false>(4 * xq, y, z, 4, g), g, p);
 }
 
-// With walls (WalledBox); XWALLS: walls on x too.
-template <typename T, bool RHO0, bool XWALLS, bool FLAT>
+// With walls (WalledBox), the cells as one sequence (BF16 256^3 with walls on all axes: 287
+// us, 335 in rectangles; FP16 with rho0 = rho 286 against 333).  XWALLS: walls on x too.
+template <typename T, bool RHO0, bool XWALLS>
 __global__ void __launch_bounds__(128, 4) k27_ab4_walls(const T *src, T *dst, Geo g, Relax27<float> p, WalledBox box)
 {
     int xq, y, z;
@@ -311,19 +314,14 @@ __global__ void __launch_bounds__(128, 4) k27_ab4_walls(const T *src, T *dst, Ge
         if (i >= box.walls.count) return;
         box.walls.at_wall(i, xq, y, z);
         ab4_body27<T, RHO0>(src, dst, Site<true>(4 * xq, y, z, 4, g), g, p);
-        return;
-    }
-    if constexpr (FLAT) {
+    } else {
         const unsigned i = box.inner_item();
         if (i >= box.inner.count) return;
         box.inner.at(i, xq, y, z);
-    } else {
-        box.inner_rectangle(xq, y, z);
-        if (xq >= (int)box.inner.per_row.d || y >= box.inner.y0 + (int)box.inner.rows.d) return;
+        Site<XWALLS> s(4 * xq, y, z, 4, g);
+        drop_yz(s);
+        ab4_body27<T, RHO0>(src, dst, s, g, p);
     }
-    Site<XWALLS> s(4 * xq, y, z, 4, g);
-    drop_yz(s);
-    ab4_body27<T, RHO0>(src, dst, s, g, p);
 }
 
 // The lattice for two FP32 steps per pass (k_pair).  16 rows leave 128 registers a
@@ -393,12 +391,17 @@ __device__ __forceinline__ void get_canonical(const T *grid, const Site<WALLS> &
     }
 }
 
-#define LBM_Q27_PROLOGUE                                    \
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;    \
-    if (i >= box.count) return;                             \
-    int x, y, z;                                            \
-    box.at(i, x, y, z);                                     \
-    const Site<true> s(x, y, z, 1, g);                      \
+// FLAT as in k27_ab1.
+#define LBM_Q27_PROLOGUE                                             \
+    int x, y, z;                                                     \
+    if (FLAT) {                                                      \
+        const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;    \
+        if (i >= box.count) return;                                  \
+        box.at(i, x, y, z);                                          \
+    } else if (!box.at_block(x, y, z)) {                             \
+        return;                                                      \
+    }                                                                \
+    const Site<true> s(x, y, z, 1, g);                               \
     const long long cell = s.own + x;
 
 // f = feq(rho, u) (Eq. 14, shifted), written in the A/B layout.
@@ -407,6 +410,7 @@ __global__ void k27_init(T *grid, const In *rho, const In *u, Geo g, Relax27<typ
                          Box box)
 {
     using R = typename Storage<T>::R;
+    constexpr bool FLAT = true;
     LBM_Q27_PROLOGUE
     const R r = rho ? R(rho[cell]) : R(1);
     const R uv[3] = {R(u[cell]), R(u[g.ncell + cell]), R(u[2 * g.ncell + cell])};
@@ -428,7 +432,7 @@ __global__ void k27_init(T *grid, const In *rho, const In *u, Geo g, Relax27<typ
     put_canonical<T, true>(grid, s, x, g, fc);
 }
 
-template <typename T, typename Out>
+template <typename T, typename Out, bool FLAT>
 __global__ void k27_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g, Relax27<typename Storage<T>::R> p,
                             int rho0_mode, Box box)
 {
@@ -450,7 +454,7 @@ __global__ void k27_moments(const T *__restrict__ grid, Out *rho, Out *u, Geo g,
         for (int i = 0; i < 3; ++i) u[i * g.ncell + cell] = Out((j[i] + p.half_a[i]) * inv);
 }
 
-template <typename T>
+template <typename T, bool FLAT>
 __global__ void k27_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g, Box box)
 {
     LBM_Q27_PROLOGUE
@@ -460,7 +464,7 @@ __global__ void k27_get(const T *__restrict__ grid, T *__restrict__ dst, Geo g, 
     for (int q = 0; q < Q27; ++q) Storage<T>::store(dst + (long long)q * g.ncell + cell, fc[q]);
 }
 
-template <typename T>
+template <typename T, bool FLAT>
 __global__ void k27_set(T *grid, const T *__restrict__ src, Geo g, Box box)
 {
     LBM_Q27_PROLOGUE
@@ -488,7 +492,21 @@ static cudaError_t q27_by_prec(int prec, F &&f)
 
 constexpr int Q27_THREADS = 256;
 static Box q27_box(const Geo &g) { return Box(g.nx, 0, g.ny, 0, g.nz); }
-static unsigned q27_blocks(const Geo &g) { return blocks_for(g.ncell, Q27_THREADS); }
+// Threads along x of blocks that are rectangles of rows, 128 where `rows` says that they
+// pay and the grid can have the rows; 0: the cells as one sequence.
+static int q27_block(const Geo &g, int threads, bool rows)
+{
+    return rows && threads % 128 == 0 && (g.ny + threads / 128 - 1) / (threads / 128) <= 65535 ? 128 : 0;
+}
+
+template <typename... P, typename... A>
+static cudaError_t launch27(void (*flat)(P...), void (*rectangles)(P...), const Geo &g, bool rows, cudaStream_t stream,
+                            A &&...args)
+{
+    const int bx = q27_block(g, Q27_THREADS, rows);
+    launch_step_box(bx ? rectangles : flat, false, q27_box(g), bx, Q27_THREADS, stream, std::forward<A>(args)...);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, const CollBoth &c, LaunchShape s,
                           cudaStream_t stream)
@@ -509,11 +527,9 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
                 auto run = [&](auto rho0, auto walled) {
                     constexpr bool RH = decltype(rho0)::value, W = decltype(walled)::value;
                     if constexpr (W) {
-                        const WalledBox box(g.nx / 4, g.nx / 4, g, QUAD_THREADS, true);
-                        const bool flat = box.bx_log2 < 0;
-                        auto k = g.wall_x ? (flat ? q27::k27_ab4_walls<T, RH, true, true> : q27::k27_ab4_walls<T, RH, true, false>)
-                                          : (flat ? q27::k27_ab4_walls<T, RH, false, true> : q27::k27_ab4_walls<T, RH, false, false>);
-                        launch_step_walls(k, false, box, QUAD_THREADS, stream, a, b, g, p);
+                        launch_step_walls(g.wall_x ? q27::k27_ab4_walls<T, RH, true> : q27::k27_ab4_walls<T, RH, false>, false,
+                                          WalledBox(g.nx / 4, g.nx / 4, g, QUAD_THREADS, false), QUAD_THREADS, stream, a, b, g,
+                                          p);
                     } else {
                         const Box box(g.nx / 4, 0, g.ny, 0, g.nz);
                         const int bx = box.block_x(QUAD_THREADS);
@@ -529,7 +545,7 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
             }
         }
         const Box box = q27_box(g);
-        const int bx = walls && s.threads >= 128 ? box.block_x(s.threads) : 0;
+        const int bx = q27_block(g, s.threads, walls && g.nx % 128 == 0);
         auto k = c.rho0_is_rho ? (bx      ? q27::k27_ab1<T, true, true, false>
                                   : walls ? q27::k27_ab1<T, true, true>
                                           : q27::k27_ab1<T, true, false>)
@@ -562,12 +578,10 @@ cudaError_t launch_init27(int prec, void *grid, const void *rho, const void *u, 
         using R = typename Storage<T>::R;
         const q27::Relax27<R> p = q27::to_relax27<R>(c);
         if (dtype == 0)
-            q27::k27_init<T, double><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
-                (T *)grid, (const double *)rho, (const double *)u, g, p, c.rho0_is_rho, q27_box(g));
-        else
-            q27::k27_init<T, float><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
-                (T *)grid, (const float *)rho, (const float *)u, g, p, c.rho0_is_rho, q27_box(g));
-        return cudaGetLastError();
+            return launch27(q27::k27_init<T, double>, q27::k27_init<T, double>, g, false, stream, (T *)grid,
+                            (const double *)rho, (const double *)u, g, p, c.rho0_is_rho);
+        return launch27(q27::k27_init<T, float>, q27::k27_init<T, float>, g, false, stream, (T *)grid, (const float *)rho,
+                        (const float *)u, g, p, c.rho0_is_rho);
     });
 }
 
@@ -579,12 +593,10 @@ cudaError_t launch_moments27(int prec, const void *grid, void *rho, void *u, int
         using R = typename Storage<T>::R;
         const q27::Relax27<R> p = q27::to_relax27<R>(c);
         if (dtype == 0)
-            q27::k27_moments<T, double><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
-                (const T *)grid, (double *)rho, (double *)u, g, p, c.rho0_is_rho, q27_box(g));
-        else
-            q27::k27_moments<T, float><<<q27_blocks(g), Q27_THREADS, 0, stream>>>(
-                (const T *)grid, (float *)rho, (float *)u, g, p, c.rho0_is_rho, q27_box(g));
-        return cudaGetLastError();
+            return launch27(q27::k27_moments<T, double, true>, q27::k27_moments<T, double, false>, g, g.nx % 128 == 0, stream,
+                            (const T *)grid, (double *)rho, (double *)u, g, p, c.rho0_is_rho);
+        return launch27(q27::k27_moments<T, float, true>, q27::k27_moments<T, float, false>, g, g.nx % 128 == 0, stream, (const T *)grid,
+                        (float *)rho, (float *)u, g, p, c.rho0_is_rho);
     });
 }
 
@@ -592,8 +604,7 @@ cudaError_t launch_get27(int prec, const void *grid, void *dst, const Geo &g, cu
 {
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        q27::k27_get<T><<<q27_blocks(g), Q27_THREADS, 0, stream>>>((const T *)grid, (T *)dst, g, q27_box(g));
-        return cudaGetLastError();
+        return launch27(q27::k27_get<T, true>, q27::k27_get<T, false>, g, g.nx % 128 == 0, stream, (const T *)grid, (T *)dst, g);
     });
 }
 
@@ -601,8 +612,10 @@ cudaError_t launch_set27(int prec, void *grid, const void *src, const Geo &g, cu
 {
     return q27_by_prec(prec, [&](auto t) {
         using T = decltype(t);
-        q27::k27_set<T><<<q27_blocks(g), Q27_THREADS, 0, stream>>>((T *)grid, (const T *)src, g, q27_box(g));
-        return cudaGetLastError();
+        // its scattered stores run faster in rectangles although those leave lanes idle
+        // (FP32: 259x307x95 327 against 274 us, 70x200x200 128 against 112; FP16 33x300x300
+        // 100 against 128)
+        return launch27(q27::k27_set<T, true>, q27::k27_set<T, false>, g, g.nx > 64, stream, (T *)grid, (const T *)src, g);
     });
 }
 

@@ -70,3 +70,19 @@ def test_in_place_16_bit_steps_beyond_l2_are_bitwise_one_cell_steps(shape, preci
         a.step(n)
         b.step(n)
         assert torch.equal(a.get_pdfs(), b.get_pdfs())
+
+
+@pytest.mark.parametrize("shape", [(128, 3, 5), (256, 5, 2), (65, 4, 3), (64, 3, 3)])
+@pytest.mark.parametrize("precision", ["f64", "f32", "f16s"])
+@pytest.mark.parametrize("walls", [(0, 0, 0), (1, 1, 1)])
+def test_d3q27_rows_in_rectangles_of_blocks(shape, precision, walls):
+    """D3Q27 steps with walls and copies of rows of whole blocks, and the set of rows longer than 64, against the
+    oracle; then a round trip through the copies."""
+    from tests.test_gpu_mapping import test_any_row_length_matches_oracle as against_oracle
+    against_oracle(shape, precision, "ab", 27, walls)
+    a = _sim(shape, precision=precision, stencil=27, equilibrium="standard", walls=tuple(bool(w) for w in walls), cells_x=1)
+    a.step(1)
+    f, m = a.get_pdfs(), a.moments(torch.float64)
+    a.set_pdfs(f)
+    assert torch.equal(a.get_pdfs(), f)
+    assert all(torch.equal(x, y) for x, y in zip(a.moments(torch.float64), m))
