@@ -144,10 +144,12 @@ struct Box {
     // Threads along x of such blocks, 128, 64 or 32 of `threads`, with the fewest
     // idle lanes at the end of a row, the larger on ties; 0: take the items as one
     // sequence, because more than 1/8 of the lanes would be idle or the grid would
-    // have too many rows.
+    // have too many rows; or because four cells an item past the row's end would pass
+    // 2^31 - 1.
     int block_x(int threads) const
     {
         const int n = (int)per_row.d;
+        if (n > (1 << 29) - 128) return 0;
         int bx = 0, idle = 0;
         for (int c = 128; c >= 32; c /= 2) {
             const int w = (n + c - 1) / c * c - n;

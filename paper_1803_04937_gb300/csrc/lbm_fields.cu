@@ -359,7 +359,7 @@ constexpr int ENS_PER_SM = 2;  // resident blocks
 // costs two more planes than it has.
 static int enstrophy_planes(const Geo &g)
 {
-    const long long columns = (long long)((g.nx + ENS_X - 1) / ENS_X) * ((g.ny + ENS_Y - 1) / ENS_Y);
+    const long long columns = (long long)((g.nx - 1) / ENS_X + 1) * ((g.ny - 1) / ENS_Y + 1);
     long long best = -1;
     int planes = g.nz;
     for (int len = 1; len <= g.nz; len += 1 + len / 16) {
@@ -418,16 +418,19 @@ __global__ void __launch_bounds__(ENS_THREADS, ENS_PER_SM)
     __shared__ R su[2][3][ENS_THREADS];
     __shared__ double sh[32];
     const int tid = threadIdx.x, lane = tid % ENS_LANES, row = tid / ENS_LANES;
-    const int ntx = (g.nx + ENS_X - 1) / ENS_X, nty = (g.ny + ENS_Y - 1) / ENS_Y, ntz = (g.nz + planes - 1) / planes;
+    const int ntx = (g.nx - 1) / ENS_X + 1, nty = (g.ny - 1) / ENS_Y + 1, ntz = (g.nz + planes - 1) / planes;
     const long long tiles = (long long)ntx * nty * ntz;
     double acc = 0.0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int tx = (int)(t % ntx), ty = (int)(t / ntx % nty), tz = (int)(t / ntx / nty);
-        const int xr = tx * ENS_X - 1 + lane, yr = ty * ENS_Y - 1 + row;
+        // one more than the thread's column and row (an edge, and the halo past it, may pass 2^31 - 1)
+        const unsigned xr = (unsigned)tx * ENS_X + lane, yr = (unsigned)ty * ENS_Y + row;
         const int z0 = tz * planes, z1 = min(z0 + planes, g.nz);
         // this thread's column, wrapped; beyond the halo it repeats some column of the lattice
-        const int x = (xr + g.nx) % g.nx, y = (yr + g.ny) % g.ny;
-        const bool own = lane >= 1 && lane <= ENS_X && row >= 1 && row <= ENS_Y && xr < g.nx && yr < g.ny;
+        const int x = (int)(((xr == 0 ? (unsigned)g.nx : xr) - 1u) % (unsigned)g.nx);
+        const int y = (int)(((yr == 0 ? (unsigned)g.ny : yr) - 1u) % (unsigned)g.ny);
+        const bool own = lane >= 1 && lane <= ENS_X && row >= 1 && row <= ENS_Y && xr <= (unsigned)g.nx &&
+                         yr <= (unsigned)g.ny;
         auto velocity = [&](int z, R u[3]) {
             R f[Q];
             gather_state<L>(P, Site<WALLS>(x, y, z < 0 ? z + g.nz : (z >= g.nz ? z - g.nz : z), 1, g), f);
