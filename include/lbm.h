@@ -265,7 +265,7 @@ int lbm_reduce(lbm_handle h, double *out);
  * bounce-back wall the ghost velocity is -u of the own cell.  Summed as lbm_reduce
  * sums, deterministic for a given lattice size.  Needs a bound scratch buffer;
  * synchronises the bound stream.  D3Q19 only.  Off the per-step path: reads every
- * population once, and those of the cells around each tile of 30 x 14 columns again.
+ * population once, and those of the cells around each tile of columns again.
  * Returns LBM_ENONFINITE if the result is not finite.
  */
 int lbm_enstrophy(lbm_handle h, double *out);

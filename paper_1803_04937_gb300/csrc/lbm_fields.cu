@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *part
 // Enstrophy 1/2 <|curl u|^2> of the state, with second-order central
 // differences of u (Eq. 17) between the axis neighbours.  Periodic axes wrap;
 // across a half-way bounce-back wall the ghost velocity is -u of the own cell
-// (the wall at rest halfway between them).  A block owns a tile of ENS_X x
-// ENS_Y columns with a halo of one and marches along z: every thread forms the
+// (the wall at rest halfway between them).  A block owns a tile of
+// columns (EnsTiles) with a halo of one and marches along z: every thread forms the
 // velocity of its column's cell once per plane, keeps those of three planes in
 // registers and shares the middle one through shared memory.  (Gathering all
 // six neighbours' populations instead took 133 loads a cell and FP64
@@ -351,26 +351,43 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double *part
 // and squared to about 70 bits (Sum): a call at 192^3 takes 238 us (657 before the tiles;
 // 190 with 48-bit terms, which fall short of FP64); FP64 storage uses FP64.  Deterministic: fixed grid,
 // fixed tiles, fixed per-thread order, fixed trees.
-constexpr int ENS_LANES = 32, ENS_ROWS = 16, ENS_THREADS = ENS_LANES * ENS_ROWS;
-constexpr int ENS_X = ENS_LANES - 2, ENS_Y = ENS_ROWS - 2;
-constexpr int ENS_PER_SM = 2;  // resident blocks
+constexpr int ENS_THREADS = 512, ENS_PER_SM = 2;  // resident blocks
+// Tile shape: 2^lanes_log2 columns along x (the halo included) and as many rows as a
+// block has threads for them: 32 columns, or another power of two where fewer tiles
+// cover the lattice (a call on 8x302x356 with 32 and now: FP32 87 and 71 us, FP64 640
+// and 319; six gathers a cell took 95 and 580).
+struct EnsTiles {
+    int lanes_log2, planes;  // planes of a tile
+    int x, y;                // columns and rows a tile owns
+};
 
-// Planes per tile: the resident blocks take the tiles in turns, and each tile
-// costs two more planes than it has.
-static int enstrophy_planes(const Geo &g)
+static EnsTiles enstrophy_tiles(const Geo &g)
 {
-    const long long columns = (long long)((g.nx - 1) / ENS_X + 1) * ((g.ny - 1) / ENS_Y + 1);
+    EnsTiles t{};
+    long long columns = -1;
+    for (const int l : {5, 4, 6, 3, 7, 2}) {
+        const int x = (1 << l) - 2, y = (ENS_THREADS >> l) - 2;
+        const long long c = (long long)((g.nx - 1) / x + 1) * ((g.ny - 1) / y + 1);
+        if (columns < 0 || c < columns) {
+            columns = c;
+            t.lanes_log2 = l;
+            t.x = x;
+            t.y = y;
+        }
+    }
+    // planes per tile: the resident blocks take the tiles in turns, and each tile costs
+    // two more planes than it has
     long long best = -1;
-    int planes = g.nz;
+    t.planes = g.nz;
     for (int len = 1; len <= g.nz; len += 1 + len / 16) {
         const long long tiles = columns * ((g.nz + len - 1) / len);
         const long long cost = (tiles + RED_SMS * ENS_PER_SM - 1) / (RED_SMS * ENS_PER_SM) * (len + 2);
         if (best < 0 || cost < best) {
             best = cost;
-            planes = len;
+            t.planes = len;
         }
     }
-    return planes;
+    return t;
 }
 
 // a - b, exact as a double-float
@@ -412,24 +429,26 @@ __device__ __forceinline__ void add_square_of_curl(Sum<double> &s, double &, dou
 
 template <typename T, int L, bool WALLS>
 __global__ void __launch_bounds__(ENS_THREADS, ENS_PER_SM)
-    k_enstrophy(Planes<T> P, double *partial, Geo g, Coll<typename Storage<T>::R> p, int planes)
+    k_enstrophy(Planes<T> P, double *partial, Geo g, Coll<typename Storage<T>::R> p, EnsTiles tile)
 {
     using R = typename Storage<T>::R;
     __shared__ R su[2][3][ENS_THREADS];
     __shared__ double sh[32];
-    const int tid = threadIdx.x, lane = tid % ENS_LANES, row = tid / ENS_LANES;
-    const int ntx = (g.nx - 1) / ENS_X + 1, nty = (g.ny - 1) / ENS_Y + 1, ntz = (g.nz + planes - 1) / planes;
+    const int lanes = 1 << tile.lanes_log2;
+    const int tid = threadIdx.x, lane = tid & (lanes - 1), row = tid >> tile.lanes_log2;
+    const int ntx = (g.nx - 1) / tile.x + 1, nty = (g.ny - 1) / tile.y + 1;
+    const int ntz = (g.nz + tile.planes - 1) / tile.planes;
     const long long tiles = (long long)ntx * nty * ntz;
     double acc = 0.0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int tx = (int)(t % ntx), ty = (int)(t / ntx % nty), tz = (int)(t / ntx / nty);
         // one more than the thread's column and row (an edge, and the halo past it, may pass 2^31 - 1)
-        const unsigned xr = (unsigned)tx * ENS_X + lane, yr = (unsigned)ty * ENS_Y + row;
-        const int z0 = tz * planes, z1 = min(z0 + planes, g.nz);
+        const unsigned xr = (unsigned)tx * tile.x + lane, yr = (unsigned)ty * tile.y + row;
+        const int z0 = tz * tile.planes, z1 = min(z0 + tile.planes, g.nz);
         // this thread's column, wrapped; beyond the halo it repeats some column of the lattice
         const int x = (int)(((xr == 0 ? (unsigned)g.nx : xr) - 1u) % (unsigned)g.nx);
         const int y = (int)(((yr == 0 ? (unsigned)g.ny : yr) - 1u) % (unsigned)g.ny);
-        const bool own = lane >= 1 && lane <= ENS_X && row >= 1 && row <= ENS_Y && xr <= (unsigned)g.nx &&
+        const bool own = lane >= 1 && lane <= tile.x && row >= 1 && row <= tile.y && xr <= (unsigned)g.nx &&
                          yr <= (unsigned)g.ny;
         auto velocity = [&](int z, R u[3]) {
             R f[Q];
@@ -456,10 +475,10 @@ __global__ void __launch_bounds__(ENS_THREADS, ENS_PER_SM)
                 const R zm0 = wzm ? -uc[0] : um[0], zm1 = wzm ? -uc[1] : um[1];
                 const R zp0 = wzp ? -uc[0] : up[0], zp1 = wzp ? -uc[1] : up[1];
                 // 2 (d_y u_z - d_z u_y), 2 (d_z u_x - d_x u_z), 2 (d_x u_y - d_y u_x)
-                add_square_of_curl(s, acc, nb(2, tid + ENS_LANES, wyp), nb(2, tid - ENS_LANES, wym), zp1, zm1);
+                add_square_of_curl(s, acc, nb(2, tid + lanes, wyp), nb(2, tid - lanes, wym), zp1, zm1);
                 add_square_of_curl(s, acc, zp0, zm0, nb(2, tid + 1, wxp), nb(2, tid - 1, wxm));
-                add_square_of_curl(s, acc, nb(1, tid + 1, wxp), nb(1, tid - 1, wxm), nb(0, tid + ENS_LANES, wyp),
-                                   nb(0, tid - ENS_LANES, wym));
+                add_square_of_curl(s, acc, nb(1, tid + 1, wxp), nb(1, tid - 1, wxm), nb(0, tid + lanes, wyp),
+                                   nb(0, tid - lanes, wym));
             }
             if ((z - z0) % SUM_CELLS == SUM_CELLS - 1) s.flush(acc);
 #pragma unroll
@@ -602,9 +621,9 @@ cudaError_t launch_enstrophy(int prec, int layout, const void *grid, double *scr
         using T = decltype(tag);
         const auto p = to_coll<typename Storage<T>::R>(c);
         const Planes<T> P = planes_of<T>(const_cast<void *>(grid), g.ncell);
-        const int planes = enstrophy_planes(g);
+        const EnsTiles tiles = enstrophy_tiles(g);
         return by_layout(layout, g, [&](auto l, auto w) {
-            k_enstrophy<T, decltype(l)::value, decltype(w)::value><<<blocks, ENS_THREADS, 0, s>>>(P, scratch, g, p, planes);
+            k_enstrophy<T, decltype(l)::value, decltype(w)::value><<<blocks, ENS_THREADS, 0, s>>>(P, scratch, g, p, tiles);
         });
     });
     if (e != cudaSuccess) return e;

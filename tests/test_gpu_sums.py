@@ -176,3 +176,14 @@ def test_umax_of_tiny_velocities(scale):
     f[1, 1, 0, 0] = f[3, 1, 0, 0] = f[5, 1, 0, 0] = 2.5 * scale  # |u| = 4.33 scale
     sim.set_pdfs(f)
     assert sim.reduce()["umax"] == pytest.approx(2.5 * scale * 3 ** 0.5, rel=1e-6, abs=0.0)
+
+
+@pytest.mark.parametrize("shape", [(4, 40, 3), (2, 70, 2), (6, 63, 4), (14, 31, 2), (62, 3, 4), (130, 2, 3), (127, 1, 2),
+                                   (1, 129, 2)])
+@pytest.mark.parametrize("walls", [(False, False, False), (True, True, False)])
+def test_enstrophy_of_every_tile_shape(shape, walls):
+    """Tiles of 4 to 128 columns, with lattices that end within and past them."""
+    sim = _sim(shape, "f32", walls=walls)
+    _random_state(sim, 3)
+    want = _curl_square_mean(sim.moments(torch.float64)[1].cpu().numpy(), walls)
+    assert abs(Fraction(sim.enstrophy()) - want) <= 40 * EPS * want
