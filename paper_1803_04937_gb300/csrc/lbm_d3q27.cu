@@ -557,7 +557,7 @@ cudaError_t launch_step27(int prec, const void *src, void *dst, const Geo &g, co
     });
 }
 
-bool pair_runs27_f32(const Geo &g, bool always) { return pair_runs<q27::Lat27>(g, always, 3.05, 3.25, 32.0); }
+bool pair_runs27_f32(const Geo &g, bool always) { return pair_runs<q27::Lat27>(g, always, {3.05, 3.0, 1.3, 32.0}); }
 
 cudaError_t launch_pair27_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t s)
 {

@@ -353,13 +353,19 @@ static inline PairTiles pair_tiles(const Geo &g, int out_rows, dim3 &grid, long 
 // Whether two steps go through k_pair.  It addresses a plane by 32-bit byte offsets
 // and forms wrapped coordinates as int, up to three edges long: a plane of 2^30 cells or
 // more, an edge above 2^29, or more tile rows than a grid may have are stepped singly
-// whatever is asked (`always`).  Otherwise where its iterations (D3Q19: 2.7 to 2.95 us
-// each, with walls 2.4 to 2.7) take less time than two one-step launches, which run
-// at `glups` from DRAM.  Not with walls on x, whose ends put half of the warps on
-// the wall path (closed box 256x192x160: 172 against 210 us), nor for lattices whose
-// grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22).
+// whatever is asked (`always`).  Otherwise where its iterations take less time than two
+// one-step launches, which run at `glups` from DRAM.  An iteration takes `us`, with walls
+// `us_walls` and the more the fewer waves overlap (D3Q19: 2.7 to 2.95 us, MRT 3.05 to
+// 3.2; with walls 3.0 in one wave, 2.7 in four, 2.4 in eight; D3Q27 with walls 4.3, 3.7
+// in three, 3.1 in nine.  With one figure for all, walled 1000x64x64 ran 98 us a step in
+// pairs, 91 singly; D3Q27 116x160x279 208 and 171).  Not with walls on x, whose ends put
+// half of the warps on the wall path (closed box 256x192x160: 172 against 210 us), nor
+// for lattices whose grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22).
+struct PairTimes {
+    double us, us_walls, us_walls_per_wave, glups;
+};
 template <typename L>
-static inline bool pair_runs(const Geo &g, bool always, double us_iteration, double us_iteration_walls, double glups)
+static inline bool pair_runs(const Geo &g, bool always, const PairTimes &t)
 {
     if ((long long)g.nx * g.ny >= 1LL << 30 || g.nx > 1 << 29 || g.ny > 1 << 29) return false;
     const bool walls = g.wall_x || g.wall_y || g.wall_z;
@@ -367,8 +373,10 @@ static inline bool pair_runs(const Geo &g, bool always, double us_iteration, dou
     long long iterations;
     pair_tiles(g, (walls ? pair_warps<L, true> : pair_warps<L, false>) - 2, grid, iterations);
     if (grid.y > 65535) return false;
-    return always || (!g.wall_x && g.ncell * 8 * L::NQ >= 200000000 &&
-                      iterations * (walls ? us_iteration_walls : us_iteration) < 2.0 * (double)g.ncell / (glups * 1e3));
+    const long long waves = ((long long)grid.x * grid.y * grid.z + PAIR_SMS - 1) / PAIR_SMS;
+    const double us = walls ? t.us_walls + t.us_walls_per_wave / waves : t.us;
+    return always ||
+           (!g.wall_x && g.ncell * 8 * L::NQ >= 200000000 && iterations * us < 2.0 * (double)g.ncell / (t.glups * 1e3));
 }
 
 template <typename L, bool RHO0, bool WALLS, bool MRT>

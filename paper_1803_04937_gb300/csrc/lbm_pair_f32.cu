@@ -3,7 +3,10 @@
 
 namespace lbm {
 
-bool pair_runs_f32(const Geo &g, bool always) { return pair_runs<Lat19>(g, always, 2.8, 2.7, 45.5); }
+bool pair_runs_f32(const Geo &g, bool always, bool mrt)
+{
+    return pair_runs<Lat19>(g, always, {mrt ? 3.1 : 2.8, 2.65, 0.3, 45.5});
+}
 
 cudaError_t launch_pair_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t s)
 {

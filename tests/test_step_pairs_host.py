@@ -82,3 +82,20 @@ def test_setting_the_reported_block_again_keeps_the_librarys_choice(nx):
     assert sim.option(_lib.OPT_STEPS_PER_PASS) == 1
     assert sim.lib.lbm_set_option(sim.h, _lib.OPT_BLOCK_Y, by) == 0
     assert sim.option(_lib.OPT_STEPS_PER_PASS) == before
+
+
+# measured on a GB300: us a step in pairs and singly
+@pytest.mark.parametrize("shape,stencil,collision,walls_y,passes", [
+    ((1000, 64, 64), 19, 0, 1, 1),     # 98.4, 91.4
+    ((512, 128, 50), 19, 0, 1, 1),     # 78.6, 73.0
+    ((171, 209, 251), 19, 0, 1, 2),    # 203.2, 210.6
+    ((85, 419, 113), 19, 0, 1, 2),     # 94.1, 98.3
+    ((512, 256, 256), 19, 1, 1, 2),    # 583, 741
+    ((96, 500, 80), 19, 2, 0, 1),      # 90.2, 86.4
+    ((300, 300, 20), 19, 2, 0, 2),     # 37.7, 41.7
+    ((256, 256, 256), 19, 2, 0, 2),    # 307, 370
+    ((116, 160, 279), 27, 1, 1, 1),    # 207.8, 170.7
+    ((171, 209, 251), 27, 1, 1, 2)])   # 295.3, 311.2
+def test_pairs_run_where_they_are_faster(shape, stencil, collision, walls_y, passes):
+    sim = _Handle(shape, stencil, options=[(_lib.OPT_COLLISION, collision), (_lib.OPT_WALLS_Y, walls_y)])
+    assert sim.option(_lib.OPT_STEPS_PER_PASS) == passes
