@@ -241,7 +241,7 @@ bool use_pairs(const lbm_ctx *h, const lbm::Geo &g)
     if (h->pairs == 0 || h->pattern != LBM_PATTERN_AB || h->precision != LBM_F32 || h->cells_x != 1 || h->block_set)
         return false;
     return h->stencil == LBM_D3Q27 ? lbm::pair_runs27_f32(g, h->pairs == 2)
-                                     : lbm::pair_runs_f32(g, h->pairs == 2, h->collision == LBM_MRT);
+                                     : lbm::pair_runs_f32(g, h->pairs == 2, h->collision == LBM_MRT, h->rho0_mode);
 }
 
 // n time steps on stream st, advancing the A/B grid `cur` or AA parity

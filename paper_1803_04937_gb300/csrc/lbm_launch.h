@@ -35,7 +35,7 @@ cudaError_t launch_step(int prec, int kind, const void *src, void *dst, const Ge
 // Two A/B steps in one pass (src -> dst), FP32 storage, D3Q19 and D3Q27; pair_runs:
 // whether they can run on this lattice and (unless always) are faster than two
 // one-step launches.
-bool pair_runs_f32(const Geo &g, bool always, bool mrt);
+bool pair_runs_f32(const Geo &g, bool always, bool mrt, bool rho0_is_rho);
 cudaError_t launch_pair_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);
 bool pair_runs27_f32(const Geo &g, bool always);
 cudaError_t launch_pair27_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t stream);

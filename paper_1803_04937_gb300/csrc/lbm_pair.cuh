@@ -357,7 +357,7 @@ static inline PairTiles pair_tiles(const Geo &g, int out_rows, dim3 &grid, long 
 // one-step launches, which run at `glups` from DRAM.  An iteration takes `us`, with walls
 // `us_walls` and the more the fewer waves overlap (D3Q19: 2.7 to 2.95 us, MRT 3.05 to
 // 3.2; with walls 3.0 in one wave, 2.7 in four, 2.4 in eight; D3Q27 with walls 4.3, 3.7
-// in three, 3.1 in nine.  With one figure for all, walled 1000x64x64 ran 98 us a step in
+// in three, 3.1 in nine; MRT with walls and rho0 = rho 3.7 in one wave.  With one figure for all, walled 1000x64x64 ran 98 us a step in
 // pairs, 91 singly; D3Q27 116x160x279 208 and 171).  Not with walls on x, whose ends put
 // half of the warps on the wall path (closed box 256x192x160: 172 against 210 us), nor
 // for lattices whose grids stay in L2 (both below 200 MB; 96^3: 20 us a step against 22).

@@ -3,9 +3,9 @@
 
 namespace lbm {
 
-bool pair_runs_f32(const Geo &g, bool always, bool mrt)
+bool pair_runs_f32(const Geo &g, bool always, bool mrt, bool rho0_is_rho)
 {
-    return pair_runs<Lat19>(g, always, {mrt ? 3.1 : 2.8, 2.65, 0.3, 45.5});
+    return pair_runs<Lat19>(g, always, {mrt ? 3.1 : 2.8, 2.65, mrt && rho0_is_rho ? 1.0 : 0.3, 45.5});
 }
 
 cudaError_t launch_pair_f32(const void *src, void *dst, const Geo &g, const CollBoth &c, cudaStream_t s)

@@ -99,3 +99,10 @@ def test_setting_the_reported_block_again_keeps_the_librarys_choice(nx):
 def test_pairs_run_where_they_are_faster(shape, stencil, collision, walls_y, passes):
     sim = _Handle(shape, stencil, options=[(_lib.OPT_COLLISION, collision), (_lib.OPT_WALLS_Y, walls_y)])
     assert sim.option(_lib.OPT_STEPS_PER_PASS) == passes
+
+
+@pytest.mark.parametrize("shape,rho0,passes", [((207, 376, 56), 1, 1), ((581, 332, 113), 0, 2)])
+def test_walled_mrt_pairs_run_where_they_are_faster(shape, rho0, passes):
+    """us a step in pairs and singly: 106.2, 96.8; 402, 531."""
+    options = [(_lib.OPT_COLLISION, _lib.MRT), (_lib.OPT_WALLS_Y, 1), (_lib.OPT_RHO0_MODE, rho0)]
+    assert _Handle(shape, options=options).option(_lib.OPT_STEPS_PER_PASS) == passes
