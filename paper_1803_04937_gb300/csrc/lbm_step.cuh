@@ -670,8 +670,13 @@ __device__ __forceinline__ void ab4_body(const Planes<T> &src, const Planes<T> &
         *reinterpret_cast<uint2 *>(reinterpret_cast<unsigned short *>(dst.p[q]) + s.own + s.x) = win[q];
 }
 
+// Blocks per SM of the periodic step: five, but four where five leave BF16 short of
+// registers (256^3: MRT 221 -> 209 us, rho0 = rho 215 -> 212; the others 7 to 20 % slower).
+template <typename T, bool RHO0, bool MRT>
+constexpr int ab4_blocks = std::is_same_v<T, __nv_bfloat16> && MRT != RHO0 ? 4 : 5;
+
 template <typename T, bool RHO0, bool MRT = false>
-__global__ void __launch_bounds__(128, 5) k_ab4(Planes<T> src, Planes<T> dst, Geo g, Relax<float> p, Box box)
+__global__ void __launch_bounds__(128, ab4_blocks<T, RHO0, MRT>) k_ab4(Planes<T> src, Planes<T> dst, Geo g, Relax<float> p, Box box)
 {
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= box.count) return;  // no lane needs another lane's data
