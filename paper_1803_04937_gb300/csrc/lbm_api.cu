@@ -564,7 +564,7 @@ int lbm_step(lbm_handle h, int n)
     if (!h->initialised) return fail(h, LBM_ESTATE, "state not initialised (lbm_init or lbm_set_pdfs)");
     const lbm::Geo g = geo(h);
     const lbm::CollBoth c = coll(h);
-    const lbm::LaunchShape shape{h->bx, h->by, h->cells_x, h->block_set ? h->bx * h->by : block_threads(h)};
+    const lbm::LaunchShape shape{h->bx, h->cells_x, h->block_set ? h->bx * h->by : block_threads(h)};
     int i = 0;
     if (h->graphs && n >= GRAPH_STEPS) {
         // Replay whole graphs of GRAPH_STEPS steps (one launch call for many

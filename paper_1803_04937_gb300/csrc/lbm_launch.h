@@ -13,7 +13,7 @@ enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_BF16 = 3 };
 
 // Layout of the current state (see lbm_device.cuh): 0 AB, 1 AA even, 2 AA odd.
 struct LaunchShape {
-    int bx, by;   // thread block of the two-cell kernels (bx along x)
+    int bx;       // LBM_OPT_BLOCK_X, of which two cells per thread need a multiple of 32
     int cells_x;  // cells per thread along x: 1, 2 (nx even) or 4 (16-bit storage, nx % 4 == 0)
     int threads;  // threads per block of the one-cell kernels
 };

@@ -862,8 +862,8 @@ __global__ void __launch_bounds__(128, MRT || WALLS ? 4 : 5)
         xq = active ? x0 >> 2 : 0;
         end = false;
     }
-    // a branch that the loads stay behind, with nothing to wait for, before the row offsets (MRT in rectangles, 256^3 FP16: 241 us a step
-    // without it, 215 with; the rho0 = rho forms are as fast without)
+    // a branch that the loads stay behind, with nothing to wait for, before the row
+    // offsets (256^3 FP16: 241 us a step without it, 215 with; with rho0 = rho no faster)
     if constexpr (FORM == ROWS_OF_BLOCKS && MRT && !RHO0 && !WALLS) {
         if (box.waits) asm volatile("griddepcontrol.wait;" ::: "memory");
     }

@@ -86,3 +86,33 @@ def test_d3q27_rows_in_rectangles_of_blocks(shape, precision, walls):
     a.set_pdfs(f)
     assert torch.equal(a.get_pdfs(), f)
     assert all(torch.equal(x, y) for x, y in zip(a.moments(torch.float64), m))
+
+
+@pytest.mark.parametrize("kw", [dict(precision="f32"), dict(precision="f16s"), dict(precision="f32", pattern="aa"),
+                                dict(precision="f16s", pattern="aa"), dict(precision="f16s", stencil=27)])
+@pytest.mark.parametrize("walls", [(False, False, False), (True, True, True)])
+def test_steps_captured_after_a_join_of_two_streams(kw, walls):
+    """Steps launched early, recorded into a caller's graph behind work of another stream and behind a plain kernel."""
+    kw = dict(kw, walls=walls, equilibrium="standard", tau=0.7)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(s1):
+        a, b = (_sim((48, 20, 12), stream=s1, **kw) for _ in range(2))
+        for sim in (a, b):
+            sim.step(2)
+        f = b.get_pdfs()
+        g = torch.zeros_like(f)
+        s1.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s1):
+            s2.wait_stream(s1)
+            with torch.cuda.stream(s2):
+                g.copy_(f)       # the populations that the steps start from pass through the other stream
+            s1.wait_stream(s2)
+            b.set_pdfs(g)
+            b.step(2)
+            g.add_(0)            # a plain kernel between the steps
+            b.step(4)
+        graph.replay()
+        a.step(6)
+        assert torch.equal(a.get_pdfs(), b.get_pdfs())
+    s1.synchronize()
