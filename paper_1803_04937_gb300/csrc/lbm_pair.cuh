@@ -21,8 +21,10 @@
 // column of the tile's inner rows.  With walls a value that crosses one is stored
 // where its reflection is read, which may be plane s + 1 of c_z = -1: 62.
 //
-// What bounds it: the issue slots (about 0.6 of them used; 400 instructions a
-// cell and step) and, next, DRAM at half the one-step traffic.  A step, one-step
+// What bounds it: latency at 24 warps per SM.  It uses 0.63 of the issue slots (413
+// instructions a cell and step) and two thirds of the copy bandwidth; the largest
+// stall is the wait for the next plane's loads (3.2 warps per issue), whose number the
+// registers cap, and the barrier of each plane follows (0.9).  A step, one-step
 // kernel -> this one: periodic 256^3 364 -> 289 us, 192^3 155 -> 131; walled
 // channel 512x256x256 739 -> 585.  Measured on the way: the loads issued after the
 // barrier 328 us at 256^3; 28 rows (72 registers) spill the prefetched plane, 364;
